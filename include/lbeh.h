@@ -191,10 +191,10 @@ int lbeh_observables(lbeh_handle *h, lbeh_obs *out);
 int lbeh_get_aux(lbeh_handle *h, int which, void *out_host);
 
 /* Time-out of the grid-barrier waits of the one-launch Poisson solves: a
- * block that polls a barrier `polls` times (about 100 ns each) without every
+ * block that polls a barrier `polls` times (an L2 round trip each) without every
  * block arriving raises an abort flag, every block returns, and the step
  * reports LBEH_ERR_BARRIER_TIMEOUT (sticky until lbeh_set_fields) instead of
- * hanging.  polls <= 0 restores the default of 2^24 (about two seconds).
+ * hanging.  polls <= 0 restores the default of 2^24 (several seconds).
  * Applies to later steps; errors: INVALID_ARG. */
 int lbeh_set_wait_limit(lbeh_handle *h, long long polls);
 

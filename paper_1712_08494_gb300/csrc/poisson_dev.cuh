@@ -519,54 +519,50 @@ __device__ void tail_vcycle(const Level<T> *__restrict__ lv, int n, int first, u
 // take the same branches.  The barrier wait is bounded: a block that gives up
 // raises an abort flag and the device status, and every block then returns.
 constexpr int kPB = 512;
-constexpr long long kSpinLimit = 1LL << 24;  // default polls of a barrier wait (~100 ns each: about two seconds)
+constexpr long long kSpinLimit = 1LL << 24;  // default polls of a barrier wait (an L2 round trip each)
 constexpr double kTrustTol = 1e-8;  // FP32 residual estimate used only above this tolerance
 constexpr double kEstErr = 1e-4;    // bound of its error relative to the last exact residual
 
 struct Bar {
-  unsigned long long arrived;  // monotonic arrival count (reset before each launch)
-  int abort, pad;
+  unsigned long long arrived;  // arrivals so far (reset before each launch); kBarAbort set: the solve gave up
 };
+constexpr unsigned long long kBarAbort = 1ull << 63;
 
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long *p) {
   unsigned long long v;
   asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ unsigned long long atom_add_acq_rel_u64(unsigned long long *p, unsigned long long v) {
-  unsigned long long o;
-  asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], %2;" : "=l"(o) : "l"(p), "l"(v) : "memory");
-  return o;
-}
-__device__ __forceinline__ int ld_acquire_s32(const int *p) {
-  int v;
-  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
+__device__ __forceinline__ void red_add_release_u64(unsigned long long *p, unsigned long long v) {
+  asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// Grid barrier: thread 0 of every block arrives with an acquire-release add
-// on a monotonic counter (releasing the block's writes, ordered by the
-// preceding __syncthreads) and polls it with acquire loads until all blocks of
-// this barrier generation have arrived.  The wait is bounded; on time-out the block raises
-// the abort flag and the status, and every block leaves at its next barrier.
-__device__ __forceinline__ bool grid_sync(Bar *bar, int *status, long long spin_limit) {
+// Grid barrier number `gen` (1, 2, ...) of a launch: thread 0 of every block
+// adds its arrival with release semantics (the block's writes, ordered by the
+// preceding __syncthreads) and polls the count with acquire loads until all
+// blocks of this generation have arrived.  What bounds it is the round trip
+// to the L2: the arrival returns no value (the target follows from the
+// generation the caller counts), the abort flag is the top bit of the polled
+// word, and polls follow each other without a sleep, so a barrier is one
+// one-way add and one load past the last arrival.  The wait is bounded; on
+// time-out the block raises the abort bit and the status, and every block
+// leaves at its next barrier.
+__device__ __forceinline__ bool grid_sync(Bar *bar, unsigned long long gen, int *status, long long spin_limit) {
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
-    const unsigned long long nb = gridDim.x;
-    const unsigned long long old = atom_add_acq_rel_u64(&bar->arrived, 1ull);
-    const unsigned long long target = (old / nb + 1) * nb;
+    const unsigned long long target = gen * gridDim.x;
+    red_add_release_u64(&bar->arrived, 1ull);
+    unsigned long long v;
     long long spins = 0;
-    while (ld_acquire_u64(&bar->arrived) < target) {
-      if (ld_acquire_s32(&bar->abort)) break;
+    while ((v = ld_acquire_u64(&bar->arrived)) < target) {  // the abort bit also ends the wait
       if (++spins > spin_limit) {
-        atomicExch(&bar->abort, 1);
+        v = atomicOr(&bar->arrived, kBarAbort) | kBarAbort;
         atomicOr(status, ST_TIMEOUT);
         break;
       }
-      __nanosleep(20);
     }
-    ok = !ld_acquire_s32(&bar->abort);
+    ok = !(v & kBarAbort);
   }
   __syncthreads();
   return ok != 0;
@@ -581,11 +577,13 @@ struct GridTeam {
   Bar *bar;
   int *status;
   long long spin_limit;  // polls of a barrier wait before the solve gives up
+  mutable unsigned long long gen = 0;  // barriers passed in this launch
+  __device__ GridTeam(Bar *b, int *s, long long limit) : bar(b), status(s), spin_limit(limit) {}
   __device__ long long rank() const { return blockIdx.x * (long long)blockDim.x + threadIdx.x; }
   __device__ long long size() const { return (long long)gridDim.x * blockDim.x; }
   __device__ int block() const { return blockIdx.x; }
   __device__ int nblocks() const { return gridDim.x; }
-  __device__ bool sync() const { return grid_sync(bar, status, spin_limit); }
+  __device__ bool sync() const { return grid_sync(bar, ++gen, status, spin_limit); }
 };
 
 struct ClusterTeam {
