@@ -64,7 +64,7 @@ template <typename T> __global__ void k_restrict(Level<T> F, Level<T> C) {
   restrict_range(F, C, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
 }
 template <typename T> __global__ void k_prolong(Level<T> F, Level<T> C) {
-  prolong_range(F, C, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
+  prolong_range<false>(F, C, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
 }
 template <typename T> __global__ void k_zero(T *p, long long n) {
   long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -358,11 +358,12 @@ __global__ void k_update_phi(double *__restrict__ phi, const T *__restrict__ x, 
 }
 
 template <typename T, bool DFM>
-__global__ void __launch_bounds__(kPB, 2) k_poisson(PArgs<T> a) {
+__global__ void __launch_bounds__(kPB, kPBlocks) k_poisson(PArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double sh[kPB];
+  __shared__ double sh[3 * kPB];
   __shared__ T sht[kPB];
-  poisson_body<T, DFM>(a, GridTeam{a.bar, a.status, a.spin_limit}, smem_raw, sh, sht);
+  __shared__ Level<T> lv[kMaxLevels];
+  poisson_body<T, DFM>(a, GridTeam{a.bar, a.status, a.spin_limit}, smem_raw, sh, sht, lv);
 }
 
 // ---------------------------------------------------------------- host
@@ -402,7 +403,6 @@ template <typename T> static bool setup(Poisson *p, const Dims &d) {
     c.N = (long long)c.nx * c.ny * c.nz;
     for (int a = 0; a < 3; ++a) {
       c.cf[a] = cf[a];
-      c.h[a] = cf[a] ? f.h[a] * T(0.25) : f.h[a];
     }
     L.push_back(c);
   }
@@ -416,6 +416,22 @@ template <typename T> static bool setup(Poisson *p, const Dims &d) {
   if (cudaFuncSetAttribute(k_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem) != cudaSuccess)
     return false;
   return true;
+}
+
+// Level table of a solve by one team: the levels above the tail are stored
+// colour by colour (1 / diag in the array the Jacobi sweeps of odd levels
+// would use); FP32 forms the finest level's faces from a colour-split copy of
+// eps, kept where its first face array would be (one array to read instead of
+// four: that level is bound by memory), FP64 stores faces and 1 / diag on
+// every level (it is bound by the FP64 rate, two operations per cycle and SM).
+template <typename T> static std::vector<Level<T>> team_table(const std::vector<Level<T>> &L, size_t ts) {
+  std::vector<Level<T>> tab(L.begin(), L.end());
+  for (size_t l = 0; l < ts; ++l) {
+    tab[l].split = true;
+    tab[l].d = tab[l].x2;
+  }
+  if (ts > 0 && std::is_same<T, float>::value) tab[0].eps = tab[0].k[0];
+  return tab;
 }
 
 template <typename T, bool DFM> static void persistent_setup(Poisson *p, const Ctx &c) {
@@ -438,13 +454,11 @@ template <typename T, bool DFM> static void persistent_setup(Poisson *p, const C
     cudaGetLastError();
     return;
   }
-  // level table in device memory; level 0 forms its face coefficients from eps
-  std::vector<Level<T>> tab(L.begin(), L.end());
-  if (ts > 0) tab[0].eps = (const T *)c.eps;
+  const std::vector<Level<T>> tab = team_table(L, ts);
   Level<T> *d = alloc<Level<T>>(p, (long long)tab.size());
   if (!d || cudaMemcpy(d, tab.data(), tab.size() * sizeof(Level<T>), cudaMemcpyHostToDevice) != cudaSuccess) return;
   p->dlevels = d;
-  p->pgrid = nsm * std::min(per, 2);
+  p->pgrid = nsm * std::min(per, kPBlocks);
   p->ptail_smem = smem;
 }
 
@@ -584,7 +598,7 @@ template <typename T> static size_t tail_start(const std::vector<Level<T>> &L) {
   size_t t = L.size() - 1;
   auto bytes = [&](size_t first) {
     size_t b = 0;
-    for (size_t l = first; l < L.size(); ++l) b += size_t(L[l].rb ? 5 : 6) * L[l].N * sizeof(T);
+    for (size_t l = first; l < L.size(); ++l) b += size_t(6) * L[l].N * sizeof(T);
     return b;
   };
   while (t > 0 && L[t - 1].N <= kTailCells && bytes(t - 1) <= kTailSmem) --t;
@@ -781,8 +795,7 @@ template <typename T, bool DFM> static long long team_setup(Poisson *p, const Ct
   for (size_t l = 0; l < L.size(); ++l) tl.L[l] = L[l];
   const size_t smem = tail_bytes(tl, (int)ts);
   if (!p->dlevels) {
-    std::vector<Level<T>> tab(L.begin(), L.end());
-    if (ts > 0) tab[0].eps = (const T *)c.eps;
+    const std::vector<Level<T>> tab = team_table(L, ts);
     Level<T> *d = alloc<Level<T>>(p, (long long)tab.size());
     if (!d || cudaMemcpy(d, tab.data(), tab.size() * sizeof(Level<T>), cudaMemcpyHostToDevice) != cudaSuccess)
       return -1;
