@@ -33,7 +33,6 @@ __global__ void __launch_bounds__(kPB, kPBlocks)
     k_batch(const BatchRec<S, T> *__restrict__ recs, int *__restrict__ par, int rec0, int nsteps) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double sh[3 * kPB];
-  __shared__ T sht[kPB];
   __shared__ Level<T> lv[kMaxLevels];
   const ClusterTeam tm;
   unsigned cid;
@@ -53,7 +52,7 @@ __global__ void __launch_bounds__(kPB, kPBlocks)
       macro_site<S, T, NC, false>(k, f, B.rho, B.J, B.psi, B.eps, B.q, n, nullptr, nullptr, nullptr, i);
     tm.sync();
     if (B.pois) {
-      poisson_body<T, DFM>(B.pa, tm, smem_raw, sh, sht, lv);
+      poisson_body<T, DFM>(B.pa, tm, smem_raw, sh, lv);
       tm.sync();
     }
     for (long long i = r0; i < N; i += G)

@@ -98,8 +98,7 @@ template <typename T> __global__ void k_coef_coarsen(Level<T> F, Level<T> C) {
 
 template <typename T> __global__ void __launch_bounds__(1024) k_tail(Tail<T> tl, int first) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ T sh[1024];
-  tail_vcycle(tl.L, tl.n, first, smem_raw, sh);
+  tail_vcycle(tl.L, tl.n, first, smem_raw);
 }
 
 // ---------------------------------------------------------------- FP64 driver kernels
@@ -361,9 +360,8 @@ template <typename T, bool DFM>
 __global__ void __launch_bounds__(kPB, kPBlocks) k_poisson(PArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double sh[3 * kPB];
-  __shared__ T sht[kPB];
   __shared__ Level<T> lv[kMaxLevels];
-  poisson_body<T, DFM>(a, GridTeam{a.bar, a.status, a.spin_limit}, smem_raw, sh, sht, lv);
+  poisson_body<T, DFM>(a, GridTeam{a.bar, a.status, a.spin_limit}, smem_raw, sh, lv);
 }
 
 // ---------------------------------------------------------------- host
@@ -426,11 +424,14 @@ template <typename T> static bool setup(Poisson *p, const Dims &d) {
 // every level (it is bound by the FP64 rate, two operations per cycle and SM).
 template <typename T> static std::vector<Level<T>> team_table(const std::vector<Level<T>> &L, size_t ts) {
   std::vector<Level<T>> tab(L.begin(), L.end());
-  for (size_t l = 0; l < ts; ++l) {
-    tab[l].split = true;
-    tab[l].d = tab[l].x2;
+  for (size_t l = 0; l < tab.size(); ++l) {
+    tab[l].split = l < ts;
+    if (tab[l].rb) tab[l].d = tab[l].x2;
   }
-  if (ts > 0 && std::is_same<T, float>::value) tab[0].eps = tab[0].k[0];
+  if (ts > 0 && std::is_same<T, float>::value) {
+    tab[0].eps = tab[0].k[0];
+    tab[0].d = nullptr;
+  }
   return tab;
 }
 

@@ -6,6 +6,7 @@
 #pragma once
 
 #include <cmath>
+#include <type_traits>
 
 #include "internal.h"
 #include "dfloat.cuh"
@@ -216,6 +217,59 @@ __device__ __forceinline__ T coarse_coef(const Level<T> &F, const Level<T> &C, i
   return cnt == 4 ? acc * T(0.25) : cnt == 2 ? acc * T(0.5) : acc;
 }
 
+// The three coarse faces of coarse cell (X, Y, Z) from the row-major eps of a
+// finest level coarsened along every axis: the eight cells inside and the two
+// planes past them along each axis are 16 loads of two cells (the general form
+// takes 72 of one); bound by its instructions (12 series of three faces).
+template <typename T>
+__device__ __forceinline__ void coarse_faces_from_eps(const T *__restrict__ eps, const Dims &f, int X, int Y, int Z,
+                                                      T (&k)[3]) {
+  using P = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
+  const unsigned nx = unsigned(f.nx), ny = unsigned(f.ny);
+  const unsigned x0 = 2u * unsigned(X), x2 = x0 + 2u == nx ? 0u : x0 + 2u;
+  unsigned y[4], z[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    y[t] = 2u * unsigned(Y) + unsigned(t);
+    if (y[t] >= ny) y[t] -= ny;
+    z[t] = 2u * unsigned(Z) + unsigned(t);
+    if (z[t] >= unsigned(f.nz)) z[t] -= unsigned(f.nz);
+  }
+  auto two = [&](unsigned x, unsigned yy, unsigned zz) -> P {
+    return *reinterpret_cast<const P *>(eps + (zz * ny + yy) * nx + x);
+  };
+  auto path = [](T e0, T e1, T e2, T e3) -> T {
+    return series(T(0.5) * (e0 + e1), T(0.5) * (e1 + e2), T(0.5) * (e2 + e3));
+  };
+  P e[2][2];  // [z][y]
+  T acc = T(0);
+#pragma unroll
+  for (int ty = 0; ty < 2; ++ty)
+#pragma unroll
+    for (int tz = 0; tz < 2; ++tz) {
+      e[tz][ty] = two(x0, y[ty], z[tz]);
+      const P n = two(x2, y[ty], z[tz]);
+      acc += path(e[tz][ty].x, e[tz][ty].y, n.x, n.y);
+    }
+  k[0] = acc * T(0.25);
+  acc = T(0);
+#pragma unroll
+  for (int tz = 0; tz < 2; ++tz) {
+    const P a2 = two(x0, y[2], z[tz]), a3 = two(x0, y[3], z[tz]);
+    acc += path(e[tz][0].x, e[tz][1].x, a2.x, a3.x);
+    acc += path(e[tz][0].y, e[tz][1].y, a2.y, a3.y);
+  }
+  k[1] = acc * T(0.25);
+  acc = T(0);
+#pragma unroll
+  for (int ty = 0; ty < 2; ++ty) {
+    const P a2 = two(x0, y[ty], z[2]), a3 = two(x0, y[ty], z[3]);
+    acc += path(e[0][ty].x, e[1][ty].x, a2.x, a3.x);
+    acc += path(e[0][ty].y, e[1][ty].y, a2.y, a3.y);
+  }
+  k[2] = acc * T(0.25);
+}
+
 // Cell t (< N/2) of one colour, colour = (x + y + z) & 1.  Red-black levels
 // have every extent even or equal to one; cells pair up along the first axis
 // of even extent.
@@ -323,6 +377,16 @@ __device__ __forceinline__ void prolong_range(const Level<T> &F, const Level<T> 
         w1[a] = T(0);
       }
     }
+    auto xc = [&](int tx, int ty, int tz) -> T {
+      const int X = tx ? I1[0] : I0[0], Y = ty ? I1[1] : I0[1], Z = tz ? I1[2] : I0[2];
+      return C.x[cell_at(C, site32(c, X, Y, Z), (X + Y + Z) & 1)];
+    };
+    T &xf = F.x[cell_at(F, unsigned(i), (x + y + z) & 1)];
+    if (C.cf[0] && C.cf[1] && C.cf[2]) {  // weights 27/64, 9/64, 3/64, 1/64
+      xf += T(0.421875) * xc(0, 0, 0) + T(0.140625) * ((xc(1, 0, 0) + xc(0, 1, 0)) + xc(0, 0, 1)) +
+            T(0.046875) * ((xc(1, 1, 0) + xc(1, 0, 1)) + xc(0, 1, 1)) + T(0.015625) * xc(1, 1, 1);
+      continue;
+    }
     T acc = T(0);
 #pragma unroll
     for (int tz = 0; tz < 2; ++tz)
@@ -332,10 +396,9 @@ __device__ __forceinline__ void prolong_range(const Level<T> &F, const Level<T> 
         for (int tx = 0; tx < 2; ++tx) {
           const T w = (tx ? w1[0] : w0[0]) * (ty ? w1[1] : w0[1]) * (tz ? w1[2] : w0[2]);
           if (w == T(0)) continue;
-          const int X = tx ? I1[0] : I0[0], Y = ty ? I1[1] : I0[1], Z = tz ? I1[2] : I0[2];
-          acc += w * C.x[cell_at(C, site32(c, X, Y, Z), (X + Y + Z) & 1)];
+          acc += w * xc(tx, ty, tz);
         }
-    F.x[cell_at(F, unsigned(i), (x + y + z) & 1)] += acc;
+    xf += acc;
   }
 }
 
@@ -420,7 +483,7 @@ template <typename T> __host__ __device__ inline size_t tail_bytes(const Tail<T>
 // bounds it is the chain of dependent half sweeps (and in FP64 the rate of
 // the one SM it runs on); see tail_smooth.
 template <typename T>
-__device__ void tail_vcycle(const Level<T> *__restrict__ lv, int n, int first, unsigned char *smem_raw, T *sh) {
+__device__ void tail_vcycle(const Level<T> *__restrict__ lv, int n, int first, unsigned char *smem_raw) {
   __shared__ Level<T> sl[kMaxLevels];
   if (threadIdx.x == 0) {
     T *p = reinterpret_cast<T *>(smem_raw);
@@ -450,12 +513,13 @@ __device__ void tail_vcycle(const Level<T> *__restrict__ lv, int n, int first, u
 #pragma unroll
       for (int a = 0; a < 3; ++a) S.k[a][i] = G.k[a][i];
       if (l == first) S.b[i] = G.b[i];
+      if (G.d) S.d[i] = G.d[i];
     }
   }
   __syncthreads();
   for (int l = first; l < n; ++l) {
     const Level<T> S = sl[l];
-    if (!S.rb) continue;
+    if (!S.rb || lv[l].d) continue;
     const Dims d = S.dims();
     for (Walk w(threadIdx.x, blockDim.x, d.nx, d.ny); w.z < d.nz; w.next()) {
       const Nbr c = nbr(d, w.u, w.y, w.z);
@@ -467,18 +531,14 @@ __device__ void tail_vcycle(const Level<T> *__restrict__ lv, int n, int first, u
   for (int l = first; l < n; ++l) {
     const Level<T> L = sl[l];
     if (l == n - 1) {
-      // coarsest: mean-free right-hand side, fixed relaxation count
-      T acc = T(0);
-      for (long long i = threadIdx.x; i < L.N; i += blockDim.x) acc += L.b[i];
-      sh[threadIdx.x] = acc;
-      __syncthreads();
-      for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-        __syncthreads();
+      // coarsest: mean-free right-hand side (one warp adds its few cells), fixed relaxation count
+      if (threadIdx.x < 32) {
+        T acc = T(0);
+        for (long long i = threadIdx.x; i < L.N; i += 32) acc += L.b[i];
+        for (int w = 16; w > 0; w >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, w);
+        const T mean = acc / T(L.N);
+        for (long long i = threadIdx.x; i < L.N; i += 32) L.b[i] -= mean;
       }
-      const T mean = sh[0] / T(L.N);
-      __syncthreads();
-      for (long long i = threadIdx.x; i < L.N; i += blockDim.x) L.b[i] -= mean;
       __syncthreads();
       tail_smooth(L, L.rb ? 4 : 30, true);
     } else {
@@ -684,16 +744,17 @@ __device__ __forceinline__ void sweep_colour(const Level<T> &L, int c, const Tea
   }
 }
 
-// 1 / diag of a split level that stores its faces
+// 1 / diag of a level that stores its faces
 template <typename T, class Team> __device__ __forceinline__ void inverse_diag(const Level<T> &L, const Team &tm) {
-  const Rows<T> r = rows_of(L);
-  const unsigned half = unsigned(L.N >> 1);
-  for (int c = 0; c < 2; ++c) {
-    const Share sh = share(tm, half);
-    for (Walk w(sh.t0, sh.dt, r.hx, r.ny); w.z < r.nz; w.next()) {
-      const Site s = split_site<1>(r, c, w.u, w.y, w.z);
-      L.d[(c ? half : 0u) + s.i] = T(1) / diag_v(faces_v<false, 1>(L, r, s, c), 0);
-    }
+  const Dims d = L.dims();
+  const Share sh = share(tm, unsigned(L.N));
+  for (Walk w(sh.t0, sh.dt, d.nx, d.ny); w.z < d.nz; w.next()) {
+    const Nbr c = nbr(d, w.u, w.y, w.z);
+    const int color = (w.u + w.y + w.z) & 1;
+    const unsigned i = cell_at(L, c.i, color);
+    // along an axis of one cell the faces are zero wherever they are read
+    const Faces<T> f = faces(L, i, cell_at(L, c.xm, color ^ 1), cell_at(L, c.ym, color ^ 1), cell_at(L, c.zm, color ^ 1));
+    L.d[i] = T(1) / ((f.xp + f.xm) + (f.yp + f.ym) + (f.zp + f.zm));
   }
 }
 
@@ -715,14 +776,22 @@ __device__ __forceinline__ void restrict_split(const Level<T> &F, const Level<T>
     const bool xrow = r.axis == 0;
     const int ry = xrow ? Y : r.axis == 1 ? Z : 0, rz = xrow ? Z : 0, j = xrow ? X : r.axis == 1 ? Y : Z;
     const int ny = xrow ? C.cf[1] : r.axis == 1 ? C.cf[2] : 0, nz = xrow ? C.cf[2] : 0;
-    for (int tz = 0; tz <= nz; ++tz)
-      for (int ty = 0; ty <= ny; ++ty) {
-        const Site s = split_site<V>(r, 0, j, ny ? 2 * ry + ty : ry, nz ? 2 * rz + tz : rz);
-        const FaceV<T, V> f = faces_v<EPS, V>(F, r, s, 0);
-        const Vec<T, V> o = off_v<V>(F, f, s, 0), x = ldv<V>(F.x + s.i), b = ldv<V>(F.b + s.i);
+    auto child_row = [&](int ty, int tz) {
+      const Site s = split_site<V>(r, 0, j, ny ? 2 * ry + ty : ry, nz ? 2 * rz + tz : rz);
+      const FaceV<T, V> f = faces_v<EPS, V>(F, r, s, 0);
+      const Vec<T, V> o = off_v<V>(F, f, s, 0), x = ldv<V>(F.x + s.i), b = ldv<V>(F.b + s.i);
 #pragma unroll
-        for (int v = 0; v < V; ++v) acc.v[v] += b.v[v] - (o.v[v] - diag_v(f, v) * x.v[v]);
-      }
+      for (int v = 0; v < V; ++v) acc.v[v] += b.v[v] - (o.v[v] - diag_v(f, v) * x.v[v]);
+    };
+    if (V == 1 && ny && nz) {  // the loads of the four child rows in flight together
+      child_row(0, 0);
+      child_row(1, 0);
+      child_row(0, 1);
+      child_row(1, 1);
+    } else {
+      for (int tz = 0; tz <= nz; ++tz)
+        for (int ty = 0; ty <= ny; ++ty) child_row(ty, tz);
+    }
     const T mean = T(1) / T(2 * (1 + ny) * (1 + nz));  // one eighth, a quarter or a half
     const unsigned I = (unsigned(Z) * unsigned(C.ny) + unsigned(Y)) * unsigned(C.nx) + unsigned(X);
 #pragma unroll
@@ -738,7 +807,10 @@ __device__ __forceinline__ void restrict_split(const Level<T> &F, const Level<T>
 template <typename T, class Team>
 __device__ __forceinline__ void restrict_to(const Level<T> &F, const Level<T> &C, const Team &tm) {
   constexpr int V = 16 / sizeof(T);
-  const bool w = F.nx > 1 && wide(F);  // coarse rows of a multiple of V cells
+  // rows of a multiple of V coarse cells, and more cells than threads: below
+  // that, one cell per thread over more SMs hides the latency of its child
+  // rows better (6.4 us with V = 2 against 3.6 at 32^3 in FP64)
+  const bool w = F.nx > 1 && wide(F) && C.N > tm.size();
   if (F.eps) {
     if (w) restrict_split<true, V>(F, C, tm);
     else restrict_split<true, 1>(F, C, tm);
@@ -762,31 +834,37 @@ __device__ __forceinline__ void prolong_black(const Level<T> &F, const Level<T> 
     const int Y0 = y >> 1, Z0 = z >> 1;
     const int Y1 = (y & 1) ? (Y0 + 1 == C.ny ? 0 : Y0 + 1) : (Y0 == 0 ? C.ny - 1 : Y0 - 1);
     const int Z1 = (z & 1) ? (Z0 + 1 == C.nz ? 0 : Z0 + 1) : (Z0 == 0 ? C.nz - 1 : Z0 - 1);
-    T g[4][V + 1];  // coarse rows (Y0, Z0), (Y1, Z0), (Y0, Z1), (Y1, Z1) at X = j - 1 + p, ...
+    // near (X0 = j + v) and far (X1) coarse cells of the coarse rows (Y0, Z0), (Y1, Z0), (Y0, Z1), (Y1, Z1)
+    const int Xe = p ? (j + V == C.nx ? 0 : j + V) : (j == 0 ? C.nx - 1 : j - 1);
+    T n[4][V], f[4][V];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int Y = (k & 1) ? Y1 : Y0, Z = (k & 2) ? Z1 : Z0;
       const unsigned row = (unsigned(Z) * cny + unsigned(Y)) * cnx;
+      const T e = C.x[cell_at(C, row + unsigned(Xe), (Xe + Y + Z) & 1)];
+      if constexpr (V == 1) {
+        n[k][0] = C.x[cell_at(C, row + unsigned(j), (j + Y + Z) & 1)];
+      } else if (C.split) {  // j is even: the V cells are V / 2 of each colour
+        const unsigned hc = unsigned(C.N >> 1), at = (row + unsigned(j)) >> 1;
+        const int q = (Y + Z) & 1;
+        const Vec<T, V / 2> ev = ldv<V / 2>(C.x + (q ? hc : 0u) + at), od = ldv<V / 2>(C.x + (q ? 0u : hc) + at);
 #pragma unroll
-      for (int v = 0; v <= V; ++v) {
-        int X = j - 1 + p + v;
-        X = X < 0 ? C.nx - 1 : X == C.nx ? 0 : X;
-        g[k][v] = C.x[cell_at(C, row + unsigned(X), (X + Y + Z) & 1)];
+        for (int v = 0; v < V; ++v) n[k][v] = (v & 1) ? od.v[v / 2] : ev.v[v / 2];
+      } else {
+        const Vec<T, V> m = ldv<V>(C.x + row + unsigned(j));
+#pragma unroll
+        for (int v = 0; v < V; ++v) n[k][v] = m.v[v];
       }
+#pragma unroll
+      for (int v = 0; v < V; ++v)
+        f[k][v] = p ? (v + 1 < V ? n[k][v + 1 < V ? v + 1 : v] : e) : (v > 0 ? n[k][v > 0 ? v - 1 : 0] : e);
     }
     T *xb = F.x + half + (unsigned(z) * unsigned(r.ny) + unsigned(y)) * unsigned(r.hx) + unsigned(j);
     Vec<T, V> x = ldv<V>(xb);
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-      T n[4], f[4];  // the near (X0) and far (X1) coarse cell of each row
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        n[k] = p ? g[k][v] : g[k][v + 1];
-        f[k] = p ? g[k][v + 1] : g[k][v];
-      }
-      x.v[v] += T(0.421875) * n[0] + T(0.140625) * ((f[0] + n[1]) + n[2]) + T(0.046875) * ((f[1] + f[2]) + n[3]) +
-                T(0.015625) * f[3];
-    }
+    for (int v = 0; v < V; ++v)
+      x.v[v] += T(0.421875) * n[0][v] + T(0.140625) * ((f[0][v] + n[1][v]) + n[2][v]) +
+                T(0.046875) * ((f[1][v] + f[2][v]) + n[3][v]) + T(0.015625) * f[3][v];
     stv<V>(xb, x);
   }
 }
@@ -1088,6 +1166,17 @@ __device__ __forceinline__ bool team_sums(double (&v)[M], double *part, const Te
   return true;
 }
 
+// FP64 scalar arithmetic (divisions, square roots) by one thread, broadcast
+// through shared memory: 512 threads repeating a relative residual took 4 us
+// a cycle at the target's FP64 rate.
+template <class F> __device__ __forceinline__ double by_one(double *cell, F f) {
+  if (threadIdx.x == 0) *cell = f();
+  __syncthreads();
+  const double v = *cell;
+  __syncthreads();
+  return v;
+}
+
 // residual pass + fixed-order sums in every block; returns false on abort
 template <typename T, bool DFM, class Team>
 __device__ bool residual_pass(const PArgs<T> &a, const Team &tm, const Level<T> &L0, double qbar, DF qbar_df,
@@ -1195,10 +1284,9 @@ __device__ __forceinline__ void carry_site(const PArgs<T> &a, const Level<T> &L,
 // the residual test and the defect-correction cycles, separated by team
 // barriers.  Every block of the team evaluates the same fixed-order sums, so
 // all blocks take the same branches.  smem_raw holds the tail levels, sh
-// (3 kPB doubles) and sht (kPB elements) block scratch, lv the level table.
+// (3 kPB doubles) block scratch, lv the level table.
 template <typename T, bool DFM, class Team>
-__device__ void poisson_body(const PArgs<T> &a, const Team &tm, unsigned char *smem_raw, double *sh, T *sht,
-                             Level<T> *lv) {
+__device__ void poisson_body(const PArgs<T> &a, const Team &tm, unsigned char *smem_raw, double *sh, Level<T> *lv) {
   // the level table in shared memory: a barrier empties the L1, and each
   // phase would begin with reads of it from the L2
   for (int l = threadIdx.x; l < a.nlev; l += blockDim.x) lv[l] = a.lv[l];
@@ -1277,29 +1365,39 @@ __device__ void poisson_body(const PArgs<T> &a, const Team &tm, unsigned char *s
   }
   double qs[1] = {sq.get()};
   if (!team_sums<1>(qs, a.part, tm, sh)) return;
-  const double qbar = qs[0] / double(N);
+  const double qbar = by_one(sh, [&] { return qs[0] / double(N); });
   const DF qbar_df = df_split(qbar);
   // coarse face coefficients, level by level, and 1 / diag of the level before
   for (int l = 1; l < a.nlev; ++l) {
     const Level<T> F = lv[l - 1], C = lv[l];
     const Dims c = C.dims();
     const Share s = share(tm, unsigned(C.N));
+    const bool from_eps = F.eps && C.cf[0] && C.cf[1] && C.cf[2] && C.nx > 1 && C.ny > 1 && C.nz > 1;
     for (Walk w(s.t0, s.dt, c.nx, c.ny); w.z < c.nz; w.next()) {
       const unsigned I = cell_at(C, site32(c, w.u, w.y, w.z), (w.u + w.y + w.z) & 1);
-      C.k[0][I] = coarse_coef<0>(F, C, w.u, w.y, w.z);
-      C.k[1][I] = coarse_coef<1>(F, C, w.u, w.y, w.z);
-      C.k[2][I] = coarse_coef<2>(F, C, w.u, w.y, w.z);
+      T k[3];
+      if (from_eps) {
+        coarse_faces_from_eps(a.eps, d, w.u, w.y, w.z, k);
+      } else {
+        k[0] = coarse_coef<0>(F, C, w.u, w.y, w.z);
+        k[1] = coarse_coef<1>(F, C, w.u, w.y, w.z);
+        k[2] = coarse_coef<2>(F, C, w.u, w.y, w.z);
+      }
+      C.k[0][I] = k[0];
+      C.k[1][I] = k[1];
+      C.k[2][I] = k[2];
     }
-    if (F.split && !F.eps) inverse_diag(F, tm);
+    if (F.d) inverse_diag(F, tm);
     if (!tm.sync()) return;
   }
+  if (lv[a.nlev - 1].d) inverse_diag(lv[a.nlev - 1], tm);  // read after the residual's barrier
   // residual test
   double r2, b2, ps;
   if (!residual_pass<T, DFM>(a, tm, L0, qbar, qbar_df, sh, r2, b2, ps)) return;
   const double tol = st->tol;
   const int max_iter = st->max_iter;
   const double bn = b2;
-  double rr = rel_res(r2, bn);
+  double rr = by_one(sh, [&] { return rel_res(r2, bn); });
   int it = 0;
   // In the FP32 modes the level-0 residual is carried from cycle to cycle in
   // FP32 (r <- r - A e); that estimate is accurate to about 1e-5 of the
@@ -1331,7 +1429,7 @@ __device__ void poisson_body(const PArgs<T> &a, const Team &tm, unsigned char *s
         restrict_to(Ll, lv[l + 1], tm);
         if (!tm.sync()) return;
       }
-      if (tm.block() == 0) tail_vcycle(lv, a.nlev, a.tail, smem_raw, sht);
+      if (tm.block() == 0) tail_vcycle(lv, a.nlev, a.tail, smem_raw);
       if (!tm.sync()) return;
       for (int l = a.tail - 1; l >= 0; --l) {
         const Level<T> Ll = lv[l];
@@ -1379,18 +1477,18 @@ __device__ void poisson_body(const PArgs<T> &a, const Team &tm, unsigned char *s
         if (!tm.sync()) return;
         if (!residual_pass<T, DFM>(a, tm, L0, qbar, qbar_df, sh, r2, b2, ps)) return;
       }
-      rr = rel_res(r2, bn);
+      rr = by_one(sh, [&] { return rel_res(r2, bn); });
       ++it;
     }
     if (exact || rr + kEstErr * rr0 < tol) break;
     if (!residual_pass<T, DFM>(a, tm, L0, qbar, qbar_df, sh, r2, b2, ps)) return;
-    rr = rel_res(r2, bn);
+    rr = by_one(sh, [&] { return rel_res(r2, bn); });
     rr0 = rr;
     exact = true;
     if (rr < tol || it >= max_iter) break;
   }
   const bool zero = bn == 0.0;
-  const double mean_phi = ps / double(N);
+  const double mean_phi = by_one(sh, [&] { return ps / double(N); });
   const DF mean_df = df_split(mean_phi);
   long long done = 0;
   if constexpr (DFM) {
