@@ -216,7 +216,7 @@ def ncu_spectral_traffic(iters_per_solve):
 
 def spectral_source_hash():
     h = hashlib.sha256()
-    for f in ("spectral.cu", "spectral.cuh", "poisson_dev.cuh", "common.cuh"):
+    for f in ("spectral_dev.cuh", "spectral.cuh", "poisson_dev.cuh", "common.cuh"):
         h.update(open(os.path.join(ROOT, "paper_1712_08494_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 

@@ -1093,7 +1093,7 @@ __device__ __forceinline__ void residual_site(const PArgs<T> &a, const Level<T> 
 // instead of 22 per cell; the thread's sums take one term per four cells.
 template <typename T>
 __device__ __forceinline__ void residual_quad(const PArgs<T> &a, const Level<T> &L0, int g, int y, int z, DF qbar,
-                                              SumAcc<true> &ar, SumAcc<true> &ab, SumAcc<true> &ap) {
+                                              float (&out)[4], float &r2, float &b2, float &ps) {
   const unsigned nx = unsigned(L0.nx), sz = nx * unsigned(L0.ny), n = unsigned(L0.N);
   const unsigned x0 = 4u * unsigned(g), row = unsigned(z) * sz + unsigned(y) * nx, i = row + x0;
   const unsigned rw[5] = {i, y + 1 == L0.ny ? i - (sz - nx) : i + nx, y == 0 ? i + (sz - nx) : i - nx,
@@ -1109,7 +1109,7 @@ __device__ __forceinline__ void residual_quad(const PArgs<T> &a, const Level<T> 
   const float hp = a.phi_hi[ip], hm = a.phi_hi[im], lp = a.phi_lo[ip], lm = a.phi_lo[im], ep = a.eps[ip],
               em = a.eps[im];
   const Vec<float, 4> q = ldv<4>(a.q + i);
-  float r2 = 0.f, b2 = 0.f, ps = 0.f, out[4];
+  r2 = b2 = ps = 0.f;
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
     const float hi[6] = {v < 3 ? h[0].v[v < 3 ? v + 1 : 3] : hp, v > 0 ? h[0].v[v > 0 ? v - 1 : 0] : hm,
@@ -1126,10 +1126,6 @@ __device__ __forceinline__ void residual_quad(const PArgs<T> &a, const Level<T> 
     b2 += r.b * r.b;
     ps += h[0].v[v];
   }
-  st_quad<float>(L0.b, unsigned(L0.N >> 1), i >> 1, (y + z) & 1, out);
-  ar.add(r2);
-  ab.add(b2);
-  ap.add(ps);
 }
 
 // Fixed-order sums of M values over the block at once: a shared-memory tree
@@ -1182,11 +1178,19 @@ template <typename T, bool DFM, class Team>
 __device__ bool residual_pass(const PArgs<T> &a, const Team &tm, const Level<T> &L0, double qbar, DF qbar_df,
                               double *sh, double &r2, double &b2, double &ps) {
   SumAcc<DFM> sr, sb, sp;
+  const long long N = L0.N;
   if constexpr (DFM) {
     if (L0.split && (L0.nx & 3) == 0) {
-      const Share s = share(tm, unsigned(L0.N >> 2));
+      const Share s = share(tm, unsigned(N >> 2));
       for (Walk w(s.t0, s.dt, L0.nx >> 2, L0.ny); w.z < L0.nz; w.next())
-        residual_quad(a, L0, w.u, w.y, w.z, qbar_df, sr, sb, sp);
+      {
+        float out[4], q2, c2, p;
+        residual_quad(a, L0, w.u, w.y, w.z, qbar_df, out, q2, c2, p);
+        st_quad<float>(L0.b, unsigned(N >> 1), site32(L0.dims(), 4 * w.u, w.y, w.z) >> 1, (w.y + w.z) & 1, out);
+        sr.add(q2);
+        sb.add(c2);
+        sp.add(p);
+      }
     } else {
       const Share s = share(tm, unsigned(L0.N));
       for (Walk w(s.t0, s.dt, L0.nx, L0.ny); w.z < L0.nz; w.next())

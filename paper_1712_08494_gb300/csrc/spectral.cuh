@@ -9,8 +9,8 @@
 // it diagonalises L with the eigenvalues
 // Lambda(k) = -sum_a 2 (1 - cos(2 pi k_a / n_a)).
 //
-// Line transforms: mixed-radix Stockham FFT (radices 8, 4, 2 with explicit
-// butterflies, 3, 5, 7 generic) of a complex line that packs two real lines
+// Line transforms: mixed-radix Stockham FFT (radices 2 to 16, butterflies with
+// compile-time roots) of a complex line that packs two real lines
 // (z = a + i b); the Hartley transforms of a and b follow from Z[k] and
 // Z[N-k]:  H_a[k] = (P[k] + M[N-k]) / 2,  H_b[k] = (M[k] - P[N-k]) / 2 with
 // P = Re Z - Im Z and M = Re Z + Im Z.
@@ -63,28 +63,69 @@ LBEH_SPEC_HD int factorize(int N, int *rad) {
   return n == 1 ? m : 0;
 }
 
-// small DFTs (forward, exp(-2 pi i / R) convention); generic for 3, 5, 7 with
-// the R-th roots taken from the line's root table w (w[t] = exp(-2 pi i t / N))
+// cos and sin of 2 pi n / d as constants: the angle's rational remainder past
+// the nearest quarter turn (at most pi/4) in a power series
+constexpr double series_cs(double x, bool sine) {
+  double t = sine ? x : 1.0, sum = t;
+  for (int k = 1; k < 12; ++k) {
+    t *= -x * x / double(sine ? (2 * k) * (2 * k + 1) : (2 * k - 1) * (2 * k));
+    sum += t;
+  }
+  return sum;
+}
+constexpr double cos_frac(int n, int d) {
+  const int q = (8 * n + d) / (2 * d);  // nearest quarter turn
+  const double x = 2.0 * 3.14159265358979323846 * double(4 * n - q * d) / double(4 * d);
+  return (q & 3) == 0 ? series_cs(x, false) : (q & 3) == 1 ? -series_cs(x, true)
+       : (q & 3) == 2 ? -series_cs(x, false) : series_cs(x, true);
+}
+constexpr double sin_frac(int n, int d) {
+  const int q = (8 * n + d) / (2 * d);
+  const double x = 2.0 * 3.14159265358979323846 * double(4 * n - q * d) / double(4 * d);
+  return (q & 3) == 0 ? series_cs(x, true) : (q & 3) == 1 ? series_cs(x, false)
+       : (q & 3) == 2 ? -series_cs(x, true) : -series_cs(x, false);
+}
+
+// Small DFTs in registers (forward, exp(-2 pi i / R) convention).  Odd primes:
+// the sums and differences of the mirrored samples times the constant cosines
+// and sines.
+template <typename T, int R, int J, int K>
+LBEH_SPEC_HD void odd_terms(C2<T> &a, C2<T> &b, const C2<T> *t, const C2<T> *d) {
+  constexpr T c = T(cos_frac((J * K) % R, R)), s = T(sin_frac((J * K) % R, R));
+  a = C2<T>{a.x + c * t[K].x, a.y + c * t[K].y};
+  b = C2<T>{b.x + s * d[K].x, b.y + s * d[K].y};
+  if constexpr (K < (R - 1) / 2) odd_terms<T, R, J, K + 1>(a, b, t, d);
+}
+template <typename T, int R, int J> LBEH_SPEC_HD void odd_rows(C2<T> *v, C2<T> v0, const C2<T> *t, const C2<T> *d) {
+  C2<T> a = v0, b{T(0), T(0)};
+  odd_terms<T, R, J, 1>(a, b, t, d);
+  v[J] = cadd(a, mul_mi(b));
+  v[R - J] = csub(a, mul_mi(b));
+  if constexpr (J < (R - 1) / 2) odd_rows<T, R, J + 1>(v, v0, t, d);
+}
 template <typename T, int R> struct Dft {
-  LBEH_SPEC_HD static void run(C2<T> *v, const C2<T> *w, int stride) {
-    C2<T> o[R];
-    for (int a = 0; a < R; ++a) {
-      C2<T> s = v[0];
-      for (int b = 1; b < R; ++b) s = cadd(s, cmul(v[b], w[((a * b) % R) * stride]));
-      o[a] = s;
+  static_assert(R == 3 || R == 5 || R == 7, "odd primes");
+  LBEH_SPEC_HD static void run(C2<T> *v) {
+    C2<T> t[(R + 1) / 2], d[(R + 1) / 2];
+    const C2<T> v0 = v[0];
+#pragma unroll
+    for (int k = 1; k <= (R - 1) / 2; ++k) {
+      t[k] = cadd(v[k], v[R - k]);
+      d[k] = csub(v[k], v[R - k]);
+      v[0] = cadd(v[0], t[k]);
     }
-    for (int a = 0; a < R; ++a) v[a] = o[a];
+    odd_rows<T, R, 1>(v, v0, t, d);
   }
 };
 template <typename T> struct Dft<T, 2> {
-  LBEH_SPEC_HD static void run(C2<T> *v, const C2<T> *, int) {
+  LBEH_SPEC_HD static void run(C2<T> *v) {
     const C2<T> a = v[0], b = v[1];
     v[0] = cadd(a, b);
     v[1] = csub(a, b);
   }
 };
 template <typename T> struct Dft<T, 4> {
-  LBEH_SPEC_HD static void run(C2<T> *v, const C2<T> *, int) {
+  LBEH_SPEC_HD static void run(C2<T> *v) {
     const C2<T> s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
     const C2<T> s13 = cadd(v[1], v[3]), d13 = mul_mi(csub(v[1], v[3]));
     v[0] = cadd(s02, s13);
@@ -94,11 +135,11 @@ template <typename T> struct Dft<T, 4> {
   }
 };
 template <typename T> struct Dft<T, 8> {
-  LBEH_SPEC_HD static void run(C2<T> *v, const C2<T> *, int) {
+  LBEH_SPEC_HD static void run(C2<T> *v) {
     // two radix-4 DFTs of the even and odd samples joined by the eighth roots
     C2<T> e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
-    Dft<T, 4>::run(e, nullptr, 0);
-    Dft<T, 4>::run(o, nullptr, 0);
+    Dft<T, 4>::run(e);
+    Dft<T, 4>::run(o);
     const T h = T(0.70710678118654752440);
     const C2<T> t1{h * (o[1].x + o[1].y), h * (o[1].y - o[1].x)};  // o1 * exp(-i pi/4)
     const C2<T> t2 = mul_mi(o[2]);                                 // o2 * exp(-i pi/2)
@@ -108,6 +149,57 @@ template <typename T> struct Dft<T, 8> {
       v[k] = cadd(e[k], t[k]);
       v[k + 4] = csub(e[k], t[k]);
     }
+  }
+};
+
+// R = A B: A-point DFTs of the samples B apart, the constant twiddles W_R^(b k), B-point DFTs across them
+template <typename T, int A, int B, int I> LBEH_SPEC_HD void const_twiddles(C2<T> (&y)[B][A]) {
+  constexpr int b = I / A, k = I % A;
+  if constexpr (b * k != 0) {
+    constexpr T c = T(cos_frac(b * k, A * B)), s = T(sin_frac(b * k, A * B));
+    y[b][k] = cmul(y[b][k], C2<T>{c, -s});
+  }
+  if constexpr (I + 1 < A * B) const_twiddles<T, A, B, I + 1>(y);
+}
+template <typename T, int A, int B> struct DftAB {
+  LBEH_SPEC_HD static void run(C2<T> *v) {
+    C2<T> y[B][A];
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+#pragma unroll
+      for (int a = 0; a < A; ++a) y[b][a] = v[B * a + b];
+      Dft<T, A>::run(y[b]);
+    }
+    const_twiddles<T, A, B, 0>(y);
+#pragma unroll
+    for (int k = 0; k < A; ++k) {
+      C2<T> t[B];
+#pragma unroll
+      for (int b = 0; b < B; ++b) t[b] = y[b][k];
+      Dft<T, B>::run(t);
+#pragma unroll
+      for (int j = 0; j < B; ++j) v[k + A * j] = t[j];
+    }
+  }
+};
+template <typename T> struct Dft<T, 6> : DftAB<T, 2, 3> {};
+template <typename T> struct Dft<T, 9> : DftAB<T, 3, 3> {};
+template <typename T> struct Dft<T, 10> : DftAB<T, 2, 5> {};
+template <typename T> struct Dft<T, 12> : DftAB<T, 4, 3> {};
+template <typename T> struct Dft<T, 14> : DftAB<T, 2, 7> {};
+template <typename T> struct Dft<T, 15> : DftAB<T, 3, 5> {};
+template <typename T> struct Dft<T, 16> : DftAB<T, 4, 4> {};
+
+// the odd primes from a table of their roots (the narrow plans below)
+template <typename T, int R> struct DftTable {
+  LBEH_SPEC_HD static void run(C2<T> *v, const C2<T> *w) {
+    C2<T> o[R];
+    for (int a = 0; a < R; ++a) {
+      C2<T> s = v[0];
+      for (int b = 1; b < R; ++b) s = cadd(s, cmul(v[b], w[(a * b) % R]));
+      o[a] = s;
+    }
+    for (int a = 0; a < R; ++a) v[a] = o[a];
   }
 };
 
@@ -121,7 +213,7 @@ LBEH_SPEC_HD void stage_bfly_r(const C2<T> *in, C2<T> *out, const C2<T> *w, int 
   const int tstep = N / (Ns * R);  // twiddle index unit of this stage
   v[0] = in[j];
   for (int r = 1; r < R; ++r) v[r] = cmul(in[j + r * stride], w[(jn * r * tstep) % N]);
-  Dft<T, R>::run(v, w, stride);
+  Dft<T, R>::run(v);
   const int idx = (j / Ns) * Ns * R + jn;
   for (int a = 0; a < R; ++a) out[idx + a * Ns] = v[a];
 }
@@ -142,40 +234,74 @@ LBEH_SPEC_HD void stage_bfly(const C2<T> *in, C2<T> *out, const C2<T> *w, int N,
 // no integer division: for stage s with radix R after sub-transforms of size
 // Ns, butterfly j (0 <= j < N/R) reads in[j + r N/R] and writes
 // out[base_j + a Ns]; code[j] packs base_j (low 16 bits) and the offset of its
-// R - 1 twiddles in the stage's twiddle table (high 16 bits).  After the
-// twiddles of a stage with a generic radix (3, 5, 7) come its R roots of unity
-// exp(-2 pi i t / R).  Radices: 8 while at least 32 butterflies remain per
-// stage, then 4, 2, 3, 5, 7.
+// R - 1 twiddles in the stage's twiddle table (high 16 bits).  A stage is a
+// pass of the line through shared memory, which is what bounds the transform,
+// so a wide plan takes as few stages as radices up to 16 allow (two up to
+// N = 225 or so), of equal size where there is a choice.  The first stage
+// stores R apart: the radix with the fewest bank conflicts goes first.  A
+// narrow plan (small boxes, whose results keep their rounding) has radices 8
+// while at least 32 butterflies remain per stage, then 4, 2, 3, 5, 7; after
+// the twiddles of its stages of radix 3, 5 and 7 come the R roots of unity.
 struct LinePlan {
   int n, nst, ncode, ntw;
   int R[kMaxStages], Ns[kMaxStages], nb[kMaxStages], code_off[kMaxStages], tw_off[kMaxStages];
+  unsigned inv[kMaxStages];  // 2^32 / nb rounded up (0: nb = 1): line of butterfly e is e inv / 2^32
+  unsigned inv_half;         // the same for N/2 + 1
+  bool wide;
 };
 
-LBEH_SPEC_HD int plan_radices(int N, int *rad) {
-  if (N < 1 || N > kMaxN) return 0;
-  int m = 0, n = N;
-  while (n % 8 == 0 && N / 8 >= 32 && m < kMaxStages) {
-    rad[m++] = 8;
-    n /= 8;
+inline bool split_radices(int n, int left, int most, int *rad) {
+  if (left == 0) return n == 1;
+  for (int r = most; r >= 2; --r) {
+    if (r == 11 || r == 13 || n % r) continue;
+    rad[left - 1] = r;
+    if (split_radices(n / r, left - 1, r, rad)) return true;
   }
-  const int order[5] = {4, 2, 3, 5, 7};
-  for (int t = 0; t < 5; ++t)
-    while (n % order[t] == 0 && m < kMaxStages) {
-      rad[m++] = order[t];
-      n /= order[t];
+  return false;
+}
+inline int plan_radices(int N, int *rad, bool wide = true) {
+  if (N < 2 || N > kMaxN) return 0;
+  if (!wide) {
+    int m = 0, n = N;
+    while (n % 8 == 0 && N / 8 >= 32 && m < kMaxStages) {
+      rad[m++] = 8;
+      n /= 8;
     }
-  return n == 1 ? m : 0;
+    const int order[5] = {4, 2, 3, 5, 7};
+    for (int t = 0; t < 5; ++t)
+      while (n % order[t] == 0 && m < kMaxStages) {
+        rad[m++] = order[t];
+        n /= order[t];
+      }
+    return n == 1 ? m : 0;
+  }
+  for (int m = 1; m <= kMaxStages; ++m)
+    for (int most = 2; most <= 16; ++most) {  // the smallest largest radix of m stages
+      if (!split_radices(N, m, most, rad)) continue;
+      auto conflicts = [](int r) { return r % 16 == 0 ? 16 : r % 8 == 0 ? 8 : r % 4 == 0 ? 4 : r % 2 == 0 ? 2 : 1; };
+      int f = 0;
+      for (int k = 1; k < m; ++k)
+        if (conflicts(rad[k]) < conflicts(rad[f]) || (conflicts(rad[k]) == conflicts(rad[f]) && rad[k] > rad[f])) f = k;
+      const int t = rad[f];
+      rad[f] = rad[0];
+      rad[0] = t;
+      return m;
+    }
+  return 0;
 }
 
 // host: the plan and its tables in FP64 (converted to the compute type by the caller)
-template <class CodeVec, class TwVec> inline bool build_plan(int N, LinePlan &P, CodeVec &code, TwVec &tw) {
+template <class CodeVec, class TwVec> inline bool build_plan(int N, LinePlan &P, CodeVec &code, TwVec &tw, bool wide = true) {
   int rad[kMaxStages];
-  const int m = plan_radices(N, rad);
+  const int m = plan_radices(N, rad, wide);
   if (!m) return false;
+  P.wide = wide;
   P.n = N;
   P.nst = m;
   code.clear();
   tw.clear();
+  auto inverse = [](int n) { return n > 1 ? unsigned((1ull << 32) / unsigned(n)) + 1u : 0u; };
+  P.inv_half = inverse(N / 2 + 1);
   const double two_pi = 6.283185307179586476925286766559;
   int Ns = 1;
   for (int s = 0; s < m; ++s) {
@@ -183,6 +309,7 @@ template <class CodeVec, class TwVec> inline bool build_plan(int N, LinePlan &P,
     P.R[s] = R;
     P.Ns[s] = Ns;
     P.nb[s] = nb;
+    P.inv[s] = inverse(nb);
     P.code_off[s] = (int)code.size();
     P.tw_off[s] = (int)tw.size();
     for (int jn = 0; jn < Ns; ++jn)
@@ -190,7 +317,7 @@ template <class CodeVec, class TwVec> inline bool build_plan(int N, LinePlan &P,
         const double a = -two_pi * double(jn * r) / double(Ns * R);
         tw.push_back({std::cos(a), std::sin(a)});
       }
-    if (R == 3 || R == 5 || R == 7)
+    if (!wide && (R == 3 || R == 5 || R == 7))
       for (int t = 0; t < R; ++t) {
         const double a = -two_pi * double(t) / double(R);
         tw.push_back({std::cos(a), std::sin(a)});
@@ -208,29 +335,59 @@ template <class CodeVec, class TwVec> inline bool build_plan(int N, LinePlan &P,
 }
 
 // butterfly j of stage s (tables of this stage: code + code_off, tw + tw_off)
-template <typename T, int R>
+template <typename T, int R, bool TABLE = false>
 LBEH_SPEC_HD void plan_bfly_r(const C2<T> *in, C2<T> *out, const C2<T> *tw, int Ns, int nb, int j, unsigned code) {
   C2<T> v[R];
   const unsigned base = code & 0xFFFFu, tb = code >> 16;
-  v[0] = in[j];
-  for (int r = 1; r < R; ++r) v[r] = cmul(in[j + r * nb], tw[tb + r - 1]);
-  Dft<T, R>::run(v, tw + Ns * (R - 1), 1);
+#pragma unroll
+  for (int r = 0; r < R; ++r) v[r] = in[j + r * nb];
+  if (Ns > 1) {
+#pragma unroll
+    for (int r = 1; r < R; ++r) v[r] = cmul(v[r], tw[tb + r - 1]);
+  }
+  if constexpr (TABLE) DftTable<T, R>::run(v, tw + Ns * (R - 1));
+  else Dft<T, R>::run(v);
+#pragma unroll
   for (int a = 0; a < R; ++a) out[base + a * Ns] = v[a];
+}
+template <bool WIDE, typename T>
+LBEH_SPEC_HD void plan_bfly_of(const LinePlan &P, int s, const unsigned *code, const C2<T> *tw, const C2<T> *in,
+                               C2<T> *out, int j) {
+  const int Ns = P.Ns[s], nb = P.nb[s];
+  const unsigned c = code[P.code_off[s] + j];
+  const C2<T> *t = tw + P.tw_off[s];
+  if constexpr (WIDE) {
+    switch (P.R[s]) {
+      case 2: plan_bfly_r<T, 2>(in, out, t, Ns, nb, j, c); break;
+      case 3: plan_bfly_r<T, 3>(in, out, t, Ns, nb, j, c); break;
+      case 4: plan_bfly_r<T, 4>(in, out, t, Ns, nb, j, c); break;
+      case 5: plan_bfly_r<T, 5>(in, out, t, Ns, nb, j, c); break;
+      case 6: plan_bfly_r<T, 6>(in, out, t, Ns, nb, j, c); break;
+      case 7: plan_bfly_r<T, 7>(in, out, t, Ns, nb, j, c); break;
+      case 8: plan_bfly_r<T, 8>(in, out, t, Ns, nb, j, c); break;
+      case 9: plan_bfly_r<T, 9>(in, out, t, Ns, nb, j, c); break;
+      case 10: plan_bfly_r<T, 10>(in, out, t, Ns, nb, j, c); break;
+      case 12: plan_bfly_r<T, 12>(in, out, t, Ns, nb, j, c); break;
+      case 14: plan_bfly_r<T, 14>(in, out, t, Ns, nb, j, c); break;
+      case 15: plan_bfly_r<T, 15>(in, out, t, Ns, nb, j, c); break;
+      default: plan_bfly_r<T, 16>(in, out, t, Ns, nb, j, c); break;
+    }
+  } else {
+    switch (P.R[s]) {
+      case 2: plan_bfly_r<T, 2>(in, out, t, Ns, nb, j, c); break;
+      case 3: plan_bfly_r<T, 3, true>(in, out, t, Ns, nb, j, c); break;
+      case 4: plan_bfly_r<T, 4>(in, out, t, Ns, nb, j, c); break;
+      case 5: plan_bfly_r<T, 5, true>(in, out, t, Ns, nb, j, c); break;
+      case 7: plan_bfly_r<T, 7, true>(in, out, t, Ns, nb, j, c); break;
+      default: plan_bfly_r<T, 8>(in, out, t, Ns, nb, j, c); break;
+    }
+  }
 }
 template <typename T>
 LBEH_SPEC_HD void plan_bfly(const LinePlan &P, int s, const unsigned *code, const C2<T> *tw, const C2<T> *in,
                             C2<T> *out, int j) {
-  const int Ns = P.Ns[s], nb = P.nb[s];
-  const unsigned c = code[P.code_off[s] + j];
-  const C2<T> *t = tw + P.tw_off[s];
-  switch (P.R[s]) {
-    case 2: plan_bfly_r<T, 2>(in, out, t, Ns, nb, j, c); break;
-    case 3: plan_bfly_r<T, 3>(in, out, t, Ns, nb, j, c); break;
-    case 4: plan_bfly_r<T, 4>(in, out, t, Ns, nb, j, c); break;
-    case 5: plan_bfly_r<T, 5>(in, out, t, Ns, nb, j, c); break;
-    case 7: plan_bfly_r<T, 7>(in, out, t, Ns, nb, j, c); break;
-    default: plan_bfly_r<T, 8>(in, out, t, Ns, nb, j, c); break;
-  }
+  if (P.wide) plan_bfly_of<true>(P, s, code, tw, in, out, j);
+  else plan_bfly_of<false>(P, s, code, tw, in, out, j);
 }
 
 // Hartley values at positions k and N-k of the two real lines packed in the

@@ -22,4 +22,10 @@ int spectral_launch_f64(Spectral *s, const Ctx &c, const PArgs<double> &pa, cuda
 int spectral_launch_f32(Spectral *s, const Ctx &c, const PArgs<float> &pa, cudaStream_t st);
 int spectral_grid(const Spectral *s);  // blocks of the launch
 
+// Kernel variants (one translation unit each: they take most of the build)
+const void *spectral_kernel_f32(bool mix);
+const void *spectral_kernel_f32_big();
+const void *spectral_kernel_f32_big_mix();
+const void *spectral_kernel_f64(bool mix);
+
 }  // namespace lbeh
