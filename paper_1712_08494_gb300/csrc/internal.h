@@ -80,8 +80,9 @@ struct PrecOps {
   // rho [ncomp][N], u [3][N] or null: device arrays, FP32 if f32 else FP64
   void (*init_eq)(Ctx &, const void *rho, const void *u, int f32);
   void (*init_f)(Ctx &, const double *f);                      // [ncomp][19][N] FP64 device
-  void (*get_f)(Ctx &, double *f);                             // [ncomp][19][N] FP64 device
-  void (*get_rho)(Ctx &, double *rho);                         // [ncomp][N] FP64 device
+  void (*get_f)(Ctx &, void *f, int f32);                      // [ncomp][19][N] FP32 / FP64 device
+  // rho of each component, ions, potential [N] and u [3][N] into device arrays (null: not wanted)
+  void (*read)(Ctx &, void *const (&out)[6], int f32);
   void (*macro)(Ctx &);
   void (*virt)(Ctx &);
   void (*collide)(Ctx &);
@@ -156,7 +157,6 @@ long long poisson_team_args(Poisson *p, const Ctx &c, void *out, size_t out_byte
 // Device buffers the solve carries from step to step (previous solution,
 // solver state): (pointer, bytes) pairs.
 void poisson_state_buffers(Poisson *p, const Ctx &c, std::vector<std::pair<void *, size_t>> &out);
-void phi_to_double(Ctx &c, double *out);       // FP64 values of the potential
 void phi_from_double(Ctx &c, const double *in);
 
 // Batched step (batch.cu; kernels in batch_<prec>.cu).

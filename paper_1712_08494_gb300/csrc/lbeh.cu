@@ -215,22 +215,10 @@ const double *stage_in(lbeh_handle *h, const void *src, int dtype, int on_device
   return out;
 }
 
-// Copy `count` FP64 device values to the caller's buffer in its dtype.
-bool stage_out(lbeh_handle *h, const double *dsrc, void *dst, int dtype, int on_device, long long count,
-               std::vector<void *> &tmp) {
-  cudaStream_t s = h->c.s;
-  if (dtype == LBEH_F64) {
-    return cuda_ok(cudaMemcpyAsync(dst, dsrc, count * 8,
-                                   on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
-  }
-  float *fd = (float *)dst;
-  if (!on_device) {
-    fd = (float *)stage_buf(h, count * 4, tmp);
-    if (!fd) return false;
-  }
-  count_launch(), k_cvt<double, float><<<grid_for(count, 256), 256, 0, s>>>(dsrc, fd, count);
-  if (!on_device) return cuda_ok(cudaMemcpyAsync(dst, fd, count * 4, cudaMemcpyDeviceToHost, s));
-  return true;
+// Copy `count` FP64 device values to the caller's FP64 buffer.
+bool stage_out(lbeh_handle *h, const double *dsrc, void *dst, int on_device, long long count) {
+  return cuda_ok(cudaMemcpyAsync(dst, dsrc, count * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                                 h->c.s));
 }
 
 // FP64 device copy of a compute-type field.
@@ -1221,7 +1209,7 @@ int lbeh_step_adjoint(lbeh_handle *h, int nsteps, int ckpt_every, const lbeh_obs
   }
   if (n0_user) {
     if (n0) {
-      if (!stage_out(h, n0, n0_user, LBEH_F64, out_dev, 2 * N, tmp)) return finish(LBEH_ERR_CUDA);
+      if (!stage_out(h, n0, n0_user, out_dev, 2 * N)) return finish(LBEH_ERR_CUDA);
     } else if (out_dev) {
       cudaMemsetAsync(n0_user, 0, 8 * 2 * N, c.s);
     } else {
@@ -1229,8 +1217,12 @@ int lbeh_step_adjoint(lbeh_handle *h, int nsteps, int ckpt_every, const lbeh_obs
     }
   }
   if (f0_user) {
-    const double *f0 = as_f64(h, fb[cur], 38 * N, tmp);
-    if (!f0 || !stage_out(h, f0, f0_user, LBEH_F64, out_dev, 38 * N, tmp)) return finish(LBEH_ERR_CUDA);
+    if (out_dev && c.prec != LBEH_FP64) {
+      count_launch(), k_cvt<float, double><<<grid_for(38 * N, 256), 256, 0, c.s>>>((const float *)fb[cur], f0_user, 38 * N);
+    } else {
+      const double *f0 = as_f64(h, fb[cur], 38 * N, tmp);
+      if (!f0 || !stage_out(h, f0, f0_user, out_dev, 38 * N)) return finish(LBEH_ERR_CUDA);
+    }
   }
   free_tmp(h, tmp);
   float ms1 = 0.f, ms2 = 0.f;
@@ -1251,35 +1243,37 @@ int lbeh_get_fields(lbeh_handle *h, lbeh_fields *out) {
   const long long N = c.d.N;
   std::vector<void *> tmp;
   bool ok = true;
-  if (out->rho[0] || out->rho[1]) {
-    double *rd = (double *)stage_buf(h, 8 * c.ncomp * N, tmp);
-    if (!rd) return LBEH_ERR_OOM;
-    h->ops.get_rho(c, rd);
-    for (int s = 0; s < c.ncomp; ++s)
-      if (out->rho[s]) ok &= stage_out(h, rd + s * N, out->rho[s], out->dtype, out->on_device, N, tmp);
+  const int f32 = out->dtype == LBEH_F32;
+  const size_t e = f32 ? 4 : 8;
+  // each wanted field goes straight to the caller's device buffer, or to a
+  // staging buffer of its element type and from there to the host
+  void *user[6] = {out->rho[0], c.ncomp == 2 ? out->rho[1] : nullptr, c.nions ? out->n[0] : nullptr,
+                   c.nions ? out->n[1] : nullptr, out->phi, out->u};
+  void *dev[6];
+  bool any = false;
+  for (int k = 0; k < 6; ++k) {
+    dev[k] = user[k];
+    if (user[k] && !out->on_device) dev[k] = stage_buf(h, e * (k == 5 ? 3 : 1) * N, tmp);
+    if (user[k] && !dev[k]) {
+      free_tmp(h, tmp);
+      return LBEH_ERR_OOM;
+    }
+    any |= user[k] != nullptr;
   }
+  if (any) h->ops.read(c, dev, f32);
+  if (!out->on_device)
+    for (int k = 0; k < 6; ++k)
+      if (user[k])
+        ok &= cuda_ok(cudaMemcpyAsync(user[k], dev[k], e * (k == 5 ? 3 : 1) * N, cudaMemcpyDeviceToHost, c.s));
   if (out->f) {
-    double *fd = nullptr;
-    fd = (decltype(fd))stage_buf(h, 8 * (size_t)c.ncomp * 19 * N, tmp);
-    if (!fd) { free_tmp(h, tmp); return LBEH_ERR_OOM; }
-    h->ops.get_f(c, fd);
-    ok &= stage_out(h, fd, out->f, out->dtype, out->on_device, (long long)c.ncomp * 19 * N, tmp);
-  }
-  if (out->u) {
-    const double *ud = as_f64(h, c.u, 3 * N, tmp);
-    ok &= ud && stage_out(h, ud, out->u, out->dtype, out->on_device, 3 * N, tmp);
-  }
-  if (c.nions) {
-    const double *nd = as_f64(h, c.n[c.ncur], 2 * N, tmp);
-    for (int s = 0; s < 2; ++s)
-      if (out->n[s]) ok &= nd && stage_out(h, nd + s * N, out->n[s], out->dtype, out->on_device, N, tmp);
-  }
-  if (out->phi) {
-    double *pd = nullptr;
-    pd = (decltype(pd))stage_buf(h, 8 * N, tmp);
-    if (!pd) { free_tmp(h, tmp); return LBEH_ERR_OOM; }
-    phi_to_double(c, pd);
-    ok &= stage_out(h, pd, out->phi, out->dtype, out->on_device, N, tmp);
+    const size_t bytes = e * c.ncomp * 19 * (size_t)N;
+    void *fd = out->on_device ? out->f : stage_buf(h, bytes, tmp);
+    if (!fd) {
+      free_tmp(h, tmp);
+      return LBEH_ERR_OOM;
+    }
+    h->ops.get_f(c, fd, f32);
+    if (!out->on_device) ok &= cuda_ok(cudaMemcpyAsync(out->f, fd, bytes, cudaMemcpyDeviceToHost, c.s));
   }
   const int nc = c.ncoll;
   if (nc && (out->cx || out->cv || out->cf)) {
@@ -1290,9 +1284,9 @@ int lbeh_get_fields(lbeh_handle *h, lbeh_fields *out) {
   if (nc && out->cq) std::memcpy(out->cq, h->hq.data(), 8 * nc);
   if (nc && out->cr) std::memcpy(out->cr, h->hr.data(), 8 * nc);
   out->ncolloid = nc;
-  const cudaError_t e = cudaGetLastError();
+  const cudaError_t err = cudaGetLastError();
   free_tmp(h, tmp);
-  if (!ok || e != cudaSuccess) return LBEH_ERR_CUDA;
+  if (!ok || err != cudaSuccess) return LBEH_ERR_CUDA;
   return LBEH_OK;
 }
 
@@ -1314,17 +1308,17 @@ int lbeh_get_aux(lbeh_handle *h, int which, void *out_host) {
     case LBEH_AUX_Q: {
       void *src = which == LBEH_AUX_PSI_S ? c.psi_s : which == LBEH_AUX_QC ? c.qc : which == LBEH_AUX_EPS ? c.eps : c.q;
       const double *d = as_f64(h, src, N, tmp);
-      ok = d && stage_out(h, d, out_host, LBEH_F64, 0, N, tmp);
+      ok = d && stage_out(h, d, out_host, 0, N);
       break;
     }
     case LBEH_AUX_RHO_V: {
       const double *d = as_f64(h, c.rho, (long long)c.ncomp * N, tmp);
-      ok = d && stage_out(h, d, out_host, LBEH_F64, 0, (long long)c.ncomp * N, tmp);
+      ok = d && stage_out(h, d, out_host, 0, (long long)c.ncomp * N);
       break;
     }
     case LBEH_AUX_U: {
       const double *d = as_f64(h, c.u, 3 * N, tmp);
-      ok = d && stage_out(h, d, out_host, LBEH_F64, 0, 3 * N, tmp);
+      ok = d && stage_out(h, d, out_host, 0, 3 * N);
       break;
     }
     default: return LBEH_ERR_INVALID_ARG;

@@ -311,12 +311,6 @@ __global__ void k_center_df(float *__restrict__ hi, float *__restrict__ lo, long
   lo[i] = v.lo;
 }
 
-__global__ void k_df_to_double(const float *__restrict__ hi, const float *__restrict__ lo, double *__restrict__ out,
-                               long long n) {
-  long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i < n) out[i] = double(hi[i]) + double(lo[i]);
-}
-
 __global__ void k_double_to_df(const double *__restrict__ in, float *__restrict__ hi, float *__restrict__ lo,
                                long long n) {
   long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -848,14 +842,7 @@ int poisson_read(Poisson *p, cudaStream_t s, PoissonStats *out) {
 }  // namespace lbeh
 
 namespace lbeh {
-// the potential as FP64 values (either representation)
-void phi_to_double(Ctx &c, double *out) {
-  if (c.prec == LBEH_FP64) {
-    cudaMemcpyAsync(out, c.phi, 8 * c.d.N, cudaMemcpyDeviceToDevice, c.s);
-  } else {
-    count_launch(), k_df_to_double<<<grid_for(c.d.N, 256), 256, 0, c.s>>>((const float *)c.phit, c.phi_lo, out, c.d.N);
-  }
-}
+// the potential from FP64 values (either representation)
 void phi_from_double(Ctx &c, const double *in) {
   if (c.prec == LBEH_FP64) {
     cudaMemcpyAsync(c.phi, in, 8 * c.d.N, cudaMemcpyDeviceToDevice, c.s);

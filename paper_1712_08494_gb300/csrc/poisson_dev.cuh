@@ -261,12 +261,16 @@ __device__ __forceinline__ void coarse_faces_from_eps(const T *__restrict__ eps,
   }
   k[1] = acc * T(0.25);
   acc = T(0);
+  P b2[2], b3[2];
 #pragma unroll
   for (int ty = 0; ty < 2; ++ty) {
-    const P a2 = two(x0, y[ty], z[2]), a3 = two(x0, y[ty], z[3]);
-    acc += path(e[0][ty].x, e[1][ty].x, a2.x, a3.x);
-    acc += path(e[0][ty].y, e[1][ty].y, a2.y, a3.y);
+    b2[ty] = two(x0, y[ty], z[2]);
+    b3[ty] = two(x0, y[ty], z[3]);
   }
+#pragma unroll
+  for (int ty = 0; ty < 2; ++ty) acc += path(e[0][ty].x, e[1][ty].x, b2[ty].x, b3[ty].x);
+#pragma unroll
+  for (int ty = 0; ty < 2; ++ty) acc += path(e[0][ty].y, e[1][ty].y, b2[ty].y, b3[ty].y);
   k[2] = acc * T(0.25);
 }
 
@@ -383,8 +387,15 @@ __device__ __forceinline__ void prolong_range(const Level<T> &F, const Level<T> 
     };
     T &xf = F.x[cell_at(F, unsigned(i), (x + y + z) & 1)];
     if (C.cf[0] && C.cf[1] && C.cf[2]) {  // weights 27/64, 9/64, 3/64, 1/64
-      xf += T(0.421875) * xc(0, 0, 0) + T(0.140625) * ((xc(1, 0, 0) + xc(0, 1, 0)) + xc(0, 0, 1)) +
-            T(0.046875) * ((xc(1, 1, 0) + xc(1, 0, 1)) + xc(0, 1, 1)) + T(0.015625) * xc(1, 1, 1);
+      T acc = T(0.421875) * xc(0, 0, 0);
+      acc += T(0.140625) * xc(1, 0, 0);
+      acc += T(0.140625) * xc(0, 1, 0);
+      acc += T(0.046875) * xc(1, 1, 0);
+      acc += T(0.140625) * xc(0, 0, 1);
+      acc += T(0.046875) * xc(1, 0, 1);
+      acc += T(0.046875) * xc(0, 1, 1);
+      acc += T(0.015625) * xc(1, 1, 1);
+      xf += acc;
       continue;
     }
     T acc = T(0);
