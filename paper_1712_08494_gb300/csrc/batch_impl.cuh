@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(kPB, kPBlocks)
     const T *n = IONS ? B.n[ncur] : nullptr;
     T *nn = IONS ? B.n[ncur ^ 1] : nullptr;
     for (long long i = r0; i < N; i += G)
-      macro_site<S, T, NC, false>(k, f, B.rho, B.J, B.psi, B.eps, B.q, n, nullptr, nullptr, nullptr, i);
+      macro_site<S, T, NC, false>(k, f, B.rho, B.J, B.psi, B.eps, B.q, n, nullptr, nullptr, nullptr, nullptr, i);
     tm.sync();
     if (B.pois) {
       poisson_body<T, DFM>(B.pa, tm, smem_raw, sh, lv);

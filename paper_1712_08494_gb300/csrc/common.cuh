@@ -96,6 +96,37 @@ __device__ __forceinline__ void coords(const Dims &d, long long i, int &x, int &
   y = int(r - zz * unsigned(d.ny));
 }
 
+// Bounding box of a sphere widened by `margin`, walked row by row (x fastest)
+// with 32-bit arithmetic: the 64-bit divisions and the signed remainders by
+// the box extents that a walk index cost before took most of the instructions
+// of the kernels that visit it.
+struct SphereBox {
+  int lo[3], cnt[3], n[3];
+  unsigned tot;
+  __device__ __forceinline__ SphereBox(const Dims &d, const double *X, double r, double margin) {
+    n[0] = d.nx;
+    n[1] = d.ny;
+    n[2] = d.nz;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const int l = int(ceil(X[a] - r - margin)), h = int(floor(X[a] + r + margin));
+      cnt[a] = max(0, min(n[a], h - l + 1));
+      lo[a] = l % n[a] + (l % n[a] < 0 ? n[a] : 0);
+    }
+    tot = unsigned(cnt[0]) * unsigned(cnt[1]) * unsigned(cnt[2]);
+  }
+  // coordinates of the t-th node (t < tot), wrapped into the box
+  __device__ __forceinline__ void node(unsigned t, int &x, int &y, int &z) const {
+    const unsigned r = t / unsigned(cnt[0]), oz = r / unsigned(cnt[1]);
+    x = lo[0] + int(t - r * unsigned(cnt[0]));
+    y = lo[1] + int(r - oz * unsigned(cnt[1]));
+    z = lo[2] + int(oz);
+    if (x >= n[0]) x -= n[0];
+    if (y >= n[1]) y -= n[1];
+    if (z >= n[2]) z -= n[2];
+  }
+};
+
 // Device status word bits (sticky until lbeh_set_fields).
 enum : int { ST_POISSON = 1, ST_NONFINITE = 2, ST_TIMEOUT = 4 };
 

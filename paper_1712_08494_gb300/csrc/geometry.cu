@@ -25,27 +25,6 @@ __device__ __forceinline__ double dist2(double px, double py, double pz, const d
   return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
 }
 
-struct Box {
-  int lo[3], cnt[3];
-};
-
-__device__ __forceinline__ Box bbox(const Dims &d, const double *X, double r, double margin) {
-  Box b;
-  const int dims[3] = {d.nx, d.ny, d.nz};
-  for (int a = 0; a < 3; ++a) {
-    b.lo[a] = int(ceil(X[a] - r - margin));
-    const int hi = int(floor(X[a] + r + margin));
-    b.cnt[a] = min(dims[a], hi - b.lo[a] + 1);
-  }
-  return b;
-}
-
-__device__ __forceinline__ void box_site(const Dims &d, const Box &b, long long t, int &x, int &y, int &z) {
-  x = ((b.lo[0] + int(t % b.cnt[0])) % d.nx + d.nx) % d.nx;
-  y = ((b.lo[1] + int((t / b.cnt[0]) % b.cnt[1])) % d.ny + d.ny) % d.ny;
-  z = ((b.lo[2] + int(t / ((long long)b.cnt[0] * b.cnt[1]))) % d.nz + d.nz) % d.nz;
-}
-
 // Position of a node or sample relative to the sphere centre, split into
 // the integer part of the centre (exact) and a fractional remainder: in FP32
 // the offset d = (x - floor(X)) + o - frac(X) is then within 1e-6 of the exact
@@ -69,8 +48,7 @@ __global__ void k_project(Dims d, int h, const double *__restrict__ cx, const do
   const double r2 = __dmul_rn(r, r);
   const float r2f = float(r2);
   const float certain = kCertain + 1e-5f * r2f;
-  const Box b = bbox(d, X, r, 1.0);
-  const long long tot = (long long)b.cnt[0] * b.cnt[1] * b.cnt[2];
+  const SphereBox b(d, X, r, 1.0);
   const int hp = h + 1;
   const double inv = double(hp) * hp * hp;
   const int dims[3] = {d.nx, d.ny, d.nz};
@@ -96,9 +74,9 @@ __global__ void k_project(Dims d, int h, const double *__restrict__ cx, const do
   const double reach = 1.7320508075688772 * (0.5 - 0.5 / double(hp)) + 1e-3;
   const double r_in = r - reach, r_out = r + reach;
   const bool shortcut = 2.0 * (r_out + 1.0) < double(min(d.nx, min(d.ny, d.nz)));
-  for (long long t = (long long)sl * blockDim.x + threadIdx.x; t < tot; t += (long long)slabs * blockDim.x) {
+  for (unsigned t = unsigned(sl) * blockDim.x + threadIdx.x; t < b.tot; t += unsigned(slabs) * blockDim.x) {
     int x, y, z;
-    box_site(d, b, t, x, y, z);
+    b.node(t, x, y, z);
     const long long i = site(d, x, y, z);
     const int p[3] = {x, y, z};
     float rel[3];
@@ -144,6 +122,34 @@ __global__ void k_project(Dims d, int h, const double *__restrict__ cx, const do
   }
 }
 
+// Nodes within r + 2 of a centre (minimum image).  A node partly covered by a
+// sphere lies within r + sqrt(3)/2 of its centre and a solid one within r, so a
+// node outside the mark has no solid D3Q19 neighbour (sqrt(2) away at most),
+// and neither it nor an axis neighbour is covered in part.  FP32 offsets carry
+// an error below 1e-4, inside the margin of 0.01.
+__global__ void k_near(Dims d, const double *__restrict__ cx, const double *__restrict__ cr, uint8_t *__restrict__ near,
+                       int slabs) {
+  const int j = blockIdx.x / slabs, sl = blockIdx.x - j * slabs;
+  const double X[3] = {cx[3 * j], cx[3 * j + 1], cx[3 * j + 2]};
+  const SphereBox b(d, X, cr[j], 2.01);
+  const int dims[3] = {d.nx, d.ny, d.nz};
+  const float lim = float(cr[j]) + 2.01f;
+  for (unsigned t = unsigned(sl) * blockDim.x + threadIdx.x; t < b.tot; t += unsigned(slabs) * blockDim.x) {
+    int p[3];
+    b.node(t, p[0], p[1], p[2]);
+    float d2 = 0.f;
+    for (int a = 0; a < 3; ++a) {
+      const double fl = floor(X[a]);
+      // the centre may lie outside the box by whole periods
+      const int rel = wrap_rel((p[a] - int(fl)) % dims[a], dims[a]);
+      float dd = fabsf(float(rel) - float(X[a] - fl));
+      dd = fminf(dd, float(dims[a]) - dd);  // the nearer image, also half a box away
+      d2 += dd * dd;
+    }
+    if (d2 < lim * lim) near[site(d, p[0], p[1], p[2])] = 1;
+  }
+}
+
 template <typename T>
 __global__ void k_surface(Dims d, const double *__restrict__ cx, const double *__restrict__ cr,
                           const uint8_t *__restrict__ solid, const int *__restrict__ owner,
@@ -151,12 +157,11 @@ __global__ void k_surface(Dims d, const double *__restrict__ cx, const double *_
                           int slabs) {
   const int j = blockIdx.x / slabs, sl = blockIdx.x - j * slabs;
   const double X[3] = {cx[3 * j], cx[3 * j + 1], cx[3 * j + 2]};
-  const Box b = bbox(d, X, cr[j], 1.0);
-  const long long tot = (long long)b.cnt[0] * b.cnt[1] * b.cnt[2];
+  const SphereBox b(d, X, cr[j], 1.0);
   int mine = 0;
-  for (long long t = (long long)sl * blockDim.x + threadIdx.x; t < tot; t += (long long)slabs * blockDim.x) {
+  for (unsigned t = unsigned(sl) * blockDim.x + threadIdx.x; t < b.tot; t += unsigned(slabs) * blockDim.x) {
     int x, y, z;
-    box_site(d, b, t, x, y, z);
+    b.node(t, x, y, z);
     const long long i = site(d, x, y, z);
     if (psi_s[i] > T(1)) psi_s[i] = T(1);
     if (!solid[i] || owner[i] != j) continue;
@@ -179,23 +184,41 @@ __global__ void k_charge(Dims d, const double *__restrict__ cx, const double *__
                          int slabs) {
   const int j = blockIdx.x / slabs, sl = blockIdx.x - j * slabs;
   const double X[3] = {cx[3 * j], cx[3 * j + 1], cx[3 * j + 2]};
-  const Box b = bbox(d, X, cr[j], 1.0);
-  const long long tot = (long long)b.cnt[0] * b.cnt[1] * b.cnt[2];
+  const SphereBox b(d, X, cr[j], 1.0);
   const double val = count[j] > 0 ? __ddiv_rn(cq[j], double(count[j])) : 0.0;
-  for (long long t = (long long)sl * blockDim.x + threadIdx.x; t < tot; t += (long long)slabs * blockDim.x) {
+  for (unsigned t = unsigned(sl) * blockDim.x + threadIdx.x; t < b.tot; t += unsigned(slabs) * blockDim.x) {
     int x, y, z;
-    box_site(d, b, t, x, y, z);
+    b.node(t, x, y, z);
     const long long i = site(d, x, y, z);
     if (surface[i] && owner[i] == j) qc[i] = T(val);
   }
 }
 
+// eight sites per thread (a byte a thread leaves the pass waiting for issue:
+// 67 us at 256^3 in FP32, where its 150 MB take 22)
 template <typename T>
-__global__ void k_psi_f(long long N, const uint8_t *__restrict__ solid, const T *__restrict__ psi_s,
-                        T *__restrict__ psi_f) {
-  long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  psi_f[i] = solid[i] ? T(0) : T(1) - psi_s[i];
+__global__ void __launch_bounds__(256) k_psi_f(long long N, const uint8_t *__restrict__ solid,
+                                               const T *__restrict__ psi_s, T *__restrict__ psi_f) {
+  const long long i = 8 * (blockIdx.x * (long long)blockDim.x + threadIdx.x);
+  if (i + 8 <= N) {
+    struct alignas(16) V {
+      T v[16 / sizeof(T)];
+    };
+    constexpr int W = 16 / sizeof(T);
+    const uint2 m = *reinterpret_cast<const uint2 *>(solid + i);
+#pragma unroll
+    for (int k = 0; k < 8; k += W) {
+      V p = *reinterpret_cast<const V *>(psi_s + i + k);
+#pragma unroll
+      for (int c = 0; c < W; ++c) {
+        const unsigned s = ((k + c < 4 ? m.x : m.y) >> (8 * ((k + c) & 3))) & 255u;
+        p.v[c] = s ? T(0) : T(1) - p.v[c];
+      }
+      *reinterpret_cast<V *>(psi_f + i + k) = p;
+    }
+    return;
+  }
+  for (long long k = i; k < N; ++k) psi_f[k] = solid[k] ? T(0) : T(1) - psi_s[k];
 }
 
 template <typename T> static void build(Ctx &c) {
@@ -205,16 +228,18 @@ template <typename T> static void build(Ctx &c) {
   cudaMemsetAsync(c.owner, 0xff, N * sizeof(int), c.s);  // -1
   cudaMemsetAsync(c.psi_s, 0, N * sizeof(T), c.s);
   cudaMemsetAsync(c.qc, 0, N * sizeof(T), c.s);
+  if (c.near) cudaMemsetAsync(c.near, 0, N, c.s);
   if (c.ncoll > 0) {
     cudaMemsetAsync(c.ccount, 0, c.ncoll * sizeof(int), c.s);
     const int sl = colloid_slabs(c.ncoll);
     count_launch(), k_project<T><<<c.ncoll * sl, 256, 0, c.s>>>(c.d, c.h, c.cx, c.cr, c.solid, c.owner, (T *)c.psi_s, sl);
+    count_launch(), k_near<<<c.ncoll * sl, 256, 0, c.s>>>(c.d, c.cx, c.cr, c.near, sl);
     count_launch(), k_surface<T><<<c.ncoll * sl, 256, 0, c.s>>>(c.d, c.cx, c.cr, c.solid, c.owner, c.surface, c.ccount,
                                                                  (T *)c.psi_s, sl);
     count_launch(), k_charge<T><<<c.ncoll * sl, 256, 0, c.s>>>(c.d, c.cx, c.cr, c.cq, c.surface, c.owner, c.ccount,
                                                                 (T *)c.qc, sl);
   }
-  count_launch(), k_psi_f<T><<<grid_for(N, 256), 256, 0, c.s>>>(N, c.solid, (const T *)c.psi_s, (T *)c.psi_f);
+  count_launch(), k_psi_f<T><<<grid_for((N + 7) / 8, 256), 256, 0, c.s>>>(N, c.solid, (const T *)c.psi_s, (T *)c.psi_f);
   c.geom_empty = c.ncoll == 0;
 }
 

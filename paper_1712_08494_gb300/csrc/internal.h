@@ -47,6 +47,7 @@ struct Ctx {
   void *flux = nullptr;    // [2][3][N]
   void *psi_s = nullptr;   // [N]
   void *psi_f = nullptr;   // [N]
+  uint8_t *near = nullptr; // [N] nodes within r + 2 of a colloid's centre (null: no colloid capacity)
   void *qc = nullptr;      // [N]
   double *phi = nullptr;   // [N] FP64 potential (FP64 mode)
   void *phit = nullptr;    // [N] potential in the compute type: aliases phi in FP64 mode; in the

@@ -486,6 +486,7 @@ int lbeh_create(const lbeh_params *p, lbeh_handle **out) {
   ok &= (c.qc = dalloc(h, T * N)) != nullptr;
   ok &= (c.solid = (uint8_t *)dalloc(h, N)) != nullptr;
   ok &= (c.surface = (uint8_t *)dalloc(h, N)) != nullptr;
+  if (p->ncolloid_max > 0) ok &= (c.near = (uint8_t *)dalloc(h, N)) != nullptr;
   ok &= (c.owner = (int *)dalloc(h, 4 * N)) != nullptr;
   if (p->nions) {
     ok &= (c.n[0] = dalloc(h, T * 2 * N)) != nullptr;
