@@ -103,6 +103,7 @@ __device__ __forceinline__ void coords(const Dims &d, long long i, int &x, int &
 struct SphereBox {
   int lo[3], cnt[3], n[3];
   unsigned tot;
+  SphereBox() = default;
   __device__ __forceinline__ SphereBox(const Dims &d, const double *X, double r, double margin) {
     n[0] = d.nx;
     n[1] = d.ny;
@@ -126,6 +127,16 @@ struct SphereBox {
     if (z >= n[2]) z -= n[2];
   }
 };
+
+// The box formed by one thread of the block: its FP64 operations, repeated by
+// every thread of the thousand blocks of a pass over the colloids, took as long
+// as the pass at the target's FP64 rate (two operations a cycle and SM).
+__device__ __forceinline__ SphereBox block_box(const Dims &d, const double *X, double r, double margin) {
+  __shared__ SphereBox b;
+  if (threadIdx.x == 0) b = SphereBox(d, X, r, margin);
+  __syncthreads();
+  return b;
+}
 
 // Device status word bits (sticky until lbeh_set_fields).
 enum : int { ST_POISSON = 1, ST_NONFINITE = 2, ST_TIMEOUT = 4 };

@@ -48,16 +48,15 @@ __global__ void k_project(Dims d, int h, const double *__restrict__ cx, const do
   const double r2 = __dmul_rn(r, r);
   const float r2f = float(r2);
   const float certain = kCertain + 1e-5f * r2f;
-  const SphereBox b(d, X, r, 1.0);
+  const SphereBox b = block_box(d, X, r, 1.0);
   const int hp = h + 1;
-  const double inv = double(hp) * hp * hp;
   const int dims[3] = {d.nx, d.ny, d.nz};
-  int Xi[3];
-  float Xf[3];
-  for (int a = 0; a < 3; ++a) {
-    const double fl = floor(X[a]);
-    Xi[a] = int(fl);
-    Xf[a] = float(X[a] - fl);  // exact difference, rounded once to FP32
+  __shared__ int Xi[3];
+  __shared__ float Xf[3];
+  if (threadIdx.x < 3) {
+    const double Xa = cx[3 * j + threadIdx.x], fl = floor(Xa);
+    Xi[threadIdx.x] = int(fl);
+    Xf[threadIdx.x] = float(Xa - fl);  // exact difference, rounded once to FP32
   }
   // sub-cube centre offsets (k + 1/2)/(h+1) - 1/2, once per block
   __shared__ double off[16];
@@ -71,9 +70,17 @@ __global__ void k_project(Dims d, int h, const double *__restrict__ cx, const do
   // a node farther than that (plus 1e-3) from the sphere surface has all its
   // samples on one side.  Used only where every sample and the node share one
   // periodic image.
-  const double reach = 1.7320508075688772 * (0.5 - 0.5 / double(hp)) + 1e-3;
-  const double r_in = r - reach, r_out = r + reach;
-  const bool shortcut = 2.0 * (r_out + 1.0) < double(min(d.nx, min(d.ny, d.nz)));
+  __shared__ float r_lim[2];  // r - reach and r + reach
+  __shared__ bool short_ok;
+  if (threadIdx.x == 0) {
+    const double reach = 1.7320508075688772 * (0.5 - 0.5 / double(hp)) + 1e-3;
+    r_lim[0] = float(r - reach);
+    r_lim[1] = float(r + reach);
+    short_ok = 2.0 * (r + reach + 1.0) < double(min(d.nx, min(d.ny, d.nz)));
+  }
+  __syncthreads();
+  const float rinf = r_lim[0], routf = r_lim[1];
+  const bool shortcut = short_ok;
   for (unsigned t = unsigned(sl) * blockDim.x + threadIdx.x; t < b.tot; t += unsigned(slabs) * blockDim.x) {
     int x, y, z;
     b.node(t, x, y, z);
@@ -93,8 +100,7 @@ __global__ void k_project(Dims d, int h, const double *__restrict__ cx, const do
       atomicMax(owner + i, j);
     }
     int nu = 0;
-    const float rinf = float(r_in), routf = float(r_out);
-    if (shortcut && r_in > 0.0 && d2f < rinf * rinf - certain) {
+    if (shortcut && rinf > 0.f && d2f < rinf * rinf - certain) {
       nu = hp * hp * hp;
     } else if (shortcut && d2f > routf * routf + certain) {
       nu = 0;
@@ -118,7 +124,8 @@ __global__ void k_project(Dims d, int h, const double *__restrict__ cx, const do
         }
       }
     }
-    if (nu) atomicAdd(psi_s + i, T(double(nu) / inv));  // dyadic values: exact in any order
+    // dyadic values: exact in any order
+    if (nu) atomicAdd(psi_s + i, nu == hp * hp * hp ? T(1) : T(double(nu) / (double(hp) * hp * hp)));
   }
 }
 
@@ -131,18 +138,26 @@ __global__ void k_near(Dims d, const double *__restrict__ cx, const double *__re
                        int slabs) {
   const int j = blockIdx.x / slabs, sl = blockIdx.x - j * slabs;
   const double X[3] = {cx[3 * j], cx[3 * j + 1], cx[3 * j + 2]};
-  const SphereBox b(d, X, cr[j], 2.01);
+  const SphereBox b = block_box(d, X, cr[j], 2.01);
   const int dims[3] = {d.nx, d.ny, d.nz};
   const float lim = float(cr[j]) + 2.01f;
+  // the centre's integer part (it may lie outside the box by whole periods) and its remainder
+  __shared__ int Xi[3];
+  __shared__ float Xf[3];
+  if (threadIdx.x < 3) {
+    const double Xa = cx[3 * j + threadIdx.x], fl = floor(Xa);
+    Xi[threadIdx.x] = int(fl);
+    Xf[threadIdx.x] = float(Xa - fl);
+  }
+  __syncthreads();
   for (unsigned t = unsigned(sl) * blockDim.x + threadIdx.x; t < b.tot; t += unsigned(slabs) * blockDim.x) {
     int p[3];
     b.node(t, p[0], p[1], p[2]);
     float d2 = 0.f;
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const double fl = floor(X[a]);
-      // the centre may lie outside the box by whole periods
-      const int rel = wrap_rel((p[a] - int(fl)) % dims[a], dims[a]);
-      float dd = fabsf(float(rel) - float(X[a] - fl));
+      const int rel = wrap_rel((p[a] - Xi[a]) % dims[a], dims[a]);
+      float dd = fabsf(float(rel) - Xf[a]);
       dd = fminf(dd, float(dims[a]) - dd);  // the nearer image, also half a box away
       d2 += dd * dd;
     }
@@ -157,7 +172,7 @@ __global__ void k_surface(Dims d, const double *__restrict__ cx, const double *_
                           int slabs) {
   const int j = blockIdx.x / slabs, sl = blockIdx.x - j * slabs;
   const double X[3] = {cx[3 * j], cx[3 * j + 1], cx[3 * j + 2]};
-  const SphereBox b(d, X, cr[j], 1.0);
+  const SphereBox b = block_box(d, X, cr[j], 1.0);
   int mine = 0;
   for (unsigned t = unsigned(sl) * blockDim.x + threadIdx.x; t < b.tot; t += unsigned(slabs) * blockDim.x) {
     int x, y, z;
@@ -184,8 +199,10 @@ __global__ void k_charge(Dims d, const double *__restrict__ cx, const double *__
                          int slabs) {
   const int j = blockIdx.x / slabs, sl = blockIdx.x - j * slabs;
   const double X[3] = {cx[3 * j], cx[3 * j + 1], cx[3 * j + 2]};
-  const SphereBox b(d, X, cr[j], 1.0);
-  const double val = count[j] > 0 ? __ddiv_rn(cq[j], double(count[j])) : 0.0;
+  const SphereBox b = block_box(d, X, cr[j], 1.0);
+  __shared__ double val;
+  if (threadIdx.x == 0) val = count[j] > 0 ? __ddiv_rn(cq[j], double(count[j])) : 0.0;
+  __syncthreads();
   for (unsigned t = unsigned(sl) * blockDim.x + threadIdx.x; t < b.tot; t += unsigned(slabs) * blockDim.x) {
     int x, y, z;
     b.node(t, x, y, z);

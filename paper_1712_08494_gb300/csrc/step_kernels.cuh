@@ -138,18 +138,18 @@ __global__ void __launch_bounds__(256) k_macro(StepK<T> k, const S *__restrict__
 }
 
 // ---------------------------------------------------------------- k_virtual
-// One block per colloid walks the colloid's bounding box; surface nodes get
+// Up to 16 blocks per colloid walk its bounding box; surface nodes get
 // the mean density of their fluid D3Q19 neighbours, and their psi and eps.
 template <typename T, int NC>
 __global__ void k_virtual(StepK<T> k, T *__restrict__ rho, T *__restrict__ psi, T *__restrict__ eps,
                           const T *__restrict__ psi_s, const uint8_t *__restrict__ solid,
                           const uint8_t *__restrict__ surface, const int *__restrict__ owner,
-                          const double *__restrict__ cx, const double *__restrict__ cr) {
-  const int j = blockIdx.x;
+                          const double *__restrict__ cx, const double *__restrict__ cr, int slabs) {
+  const int j = blockIdx.x / slabs, sl = blockIdx.x - j * slabs;
   const Dims d = k.d;
   const long long N = d.N;
-  const SphereBox box(d, cx + 3 * j, cr[j], 2.0);
-  for (unsigned t = threadIdx.x; t < box.tot; t += blockDim.x) {
+  const SphereBox box = block_box(d, cx + 3 * j, cr[j], 2.0);
+  for (unsigned t = unsigned(sl) * blockDim.x + threadIdx.x; t < box.tot; t += unsigned(slabs) * blockDim.x) {
     int x, y, z;
     box.node(t, x, y, z);
     long long i = site(d, x, y, z);
@@ -784,10 +784,6 @@ __global__ void __launch_bounds__(kObsChunk) k_obs(StepK<T> k, const S *__restri
 // What bounds the kernel is FP64 issue (two lanes a cycle): direction by
 // direction, a handful of the 32 lanes had a link, and the products of all 18
 // directions were issued for them.
-__device__ __forceinline__ long long nb_of(const Dims &d, int x, int y, int z, int q) {
-  const int xx = x + cx(q), yy = y + cy(q), zz = z + cz(q);
-  return site(d, wrap(xx, d.nx), wrap(yy, d.ny), wrap(zz, d.nz));
-}
 template <typename S, typename T, int NC>
 __global__ void __launch_bounds__(256) k_colloid_bb(
     StepK<T> k, const S *__restrict__ fn, const T *__restrict__ rhoF, const uint8_t *__restrict__ solid,
@@ -797,7 +793,7 @@ __global__ void __launch_bounds__(256) k_colloid_bb(
   const int j = blockIdx.x;
   const Dims d = k.d;
   const long long N = d.N;
-  const SphereBox box(d, ccx + 3 * j, ccr[j], 2.0);
+  const SphereBox box = block_box(d, ccx + 3 * j, ccr[j], 2.0);
   __shared__ double cvd_of[19];          // colloid velocity along each link
   __shared__ double c_of[19][3];         // the links
   __shared__ double dps[8][32 * 18];     // exchange of the links of each warp's 32 nodes
@@ -832,9 +828,13 @@ __global__ void __launch_bounds__(256) k_colloid_bb(
       } else {
 #pragma unroll
         for (int qd = 1; qd < 19; ++qd) links |= solid[nb[qd]] ? 1u << (qd - 1) : 0u;
-        for (unsigned m = links; m; m &= m - 1) {
-          const int b = __ffs(m) - 1;
-          if (owner[nb_of(d, x, y, z, b + 1)] != j) links &= ~(1u << b);
+        if (links) {  // the owners' loads in flight together
+          int own[18];
+#pragma unroll
+          for (int b = 0; b < 18; ++b) own[b] = (links >> b & 1u) ? owner[nb[b + 1]] : j;
+#pragma unroll
+          for (int b = 0; b < 18; ++b)
+            if (own[b] != j) links &= ~(1u << b);
         }
       }
     }
@@ -912,7 +912,7 @@ __global__ void k_remap(StepK<T> k, S *__restrict__ f, const uint8_t *__restrict
   const int j = blockIdx.x;
   const Dims d = k.d;
   const long long N = d.N;
-  const SphereBox box(d, ccx + 3 * j, ccr[j], 3.0);
+  const SphereBox box = block_box(d, ccx + 3 * j, ccr[j], 3.0);
   const double v[3] = {cv[3 * j], cv[3 * j + 1], cv[3 * j + 2]};
   double acc[3] = {0, 0, 0};
   for (unsigned t = threadIdx.x; t < box.tot; t += blockDim.x) {
@@ -970,7 +970,7 @@ __global__ void k_remap(StepK<T> k, S *__restrict__ f, const uint8_t *__restrict
 
 // Ions of covered nodes go in equal shares to their D3Q19 neighbours that are
 // fluid before and after the move.  Pass 1 (one block per colloid, its new
-// bounding box): each covered node stores its share n/m (m kept neighbours),
+// bounding box: over 16 blocks it took 35 us instead of 23): each covered node stores its share n/m (m kept neighbours),
 // clears its own ions and flags its kept neighbours.  Pass 2 (whole lattice,
 // a flag byte per site): flagged nodes gather the shares of their covered
 // neighbours in a fixed order and clear the flag.
@@ -982,7 +982,7 @@ __global__ void k_remap_mark(StepK<T> k, T *__restrict__ n, const uint8_t *__res
   const int j = blockIdx.x;
   const Dims d = k.d;
   const long long N = d.N;
-  const SphereBox box(d, ccx + 3 * j, ccr[j], 2.0);
+  const SphereBox box = block_box(d, ccx + 3 * j, ccr[j], 2.0);
   for (unsigned t = threadIdx.x; t < box.tot; t += blockDim.x) {
     int x, y, z;
     box.node(t, x, y, z);
@@ -1102,12 +1102,13 @@ template <typename S, typename T> struct Launch {
   static void virt(Ctx &c) {
     if (!c.solids || c.ncoll == 0) return;
     auto k = make_stepk<T>(c);
+    const int sl = colloid_slabs(c.ncoll);
     if (c.ncomp == 2)
-      count_launch(), k_virtual<T, 2><<<c.ncoll, B, 0, c.s>>>(k, (T *)c.rho, (T *)c.psi, (T *)c.eps, (const T *)c.psi_s, c.solid,
-                                              c.surface, c.owner, c.cx, c.cr);
+      count_launch(), k_virtual<T, 2><<<c.ncoll * sl, B, 0, c.s>>>(k, (T *)c.rho, (T *)c.psi, (T *)c.eps, (const T *)c.psi_s, c.solid,
+                                              c.surface, c.owner, c.cx, c.cr, sl);
     else
-      count_launch(), k_virtual<T, 1><<<c.ncoll, B, 0, c.s>>>(k, (T *)c.rho, (T *)c.psi, (T *)c.eps, (const T *)c.psi_s, c.solid,
-                                              c.surface, c.owner, c.cx, c.cr);
+      count_launch(), k_virtual<T, 1><<<c.ncoll * sl, B, 0, c.s>>>(k, (T *)c.rho, (T *)c.psi, (T *)c.eps, (const T *)c.psi_s, c.solid,
+                                              c.surface, c.owner, c.cx, c.cr, sl);
   }
   template <int NC, bool SOL, bool IONS> static void collide_v(Ctx &c) {
     auto k = make_stepk<T>(c);
