@@ -71,18 +71,63 @@ __device__ __forceinline__ void nb6(const Dims &d, long long i, long long jp[3],
   jm[2] = site(d, x, y, wrapm(z, d.nz));
 }
 
-// E at site j (central difference of phi plus the applied field)
+// 32-bit neighbour indices of a site from its periodic offsets along each axis
+// (boxes below 2^31 sites): the 19 64-bit indices of a site and a coordinate
+// decomposition for each neighbour's field took more instructions than the
+// transposes themselves (ak_a 337 us of a 96^3 step, at its 128 registers).
+struct Nb32 {
+  int i, x, y, z, nx, ny, nz;
+  int oxp, oxm, oyp, oym, ozp, ozm;
+  __device__ __forceinline__ Nb32(const Dims &d, int site) : i(site), nx(d.nx), ny(d.ny), nz(d.nz) {
+    const unsigned r = unsigned(i) / unsigned(nx);
+    x = i - int(r) * nx;
+    z = int(r / unsigned(ny));
+    y = int(r) - z * ny;
+    const int nxy = nx * ny;
+    oxp = x + 1 == nx ? 1 - nx : 1;
+    oxm = x == 0 ? nx - 1 : -1;
+    oyp = y + 1 == ny ? (1 - ny) * nx : nx;
+    oym = y == 0 ? (ny - 1) * nx : -nx;
+    ozp = z + 1 == nz ? (1 - nz) * nxy : nxy;
+    ozm = z == 0 ? (nz - 1) * nxy : -nxy;
+  }
+  __device__ __forceinline__ int operator[](int q) const {
+    return i + (cx(q) < 0 ? oxm : (cx(q) > 0 ? oxp : 0)) + (cy(q) < 0 ? oym : (cy(q) > 0 ? oyp : 0)) +
+           (cz(q) < 0 ? ozm : (cz(q) > 0 ? ozp : 0));
+  }
+  __device__ __forceinline__ int p(int a) const { return i + (a == 0 ? oxp : a == 1 ? oyp : ozp); }
+  __device__ __forceinline__ int m(int a) const { return i + (a == 0 ? oxm : a == 1 ? oym : ozm); }
+  // two sites away along an axis
+  __device__ __forceinline__ int p2(int a) const {
+    if (a == 0) return i + (x + 2 >= nx ? 2 - nx : 2);
+    if (a == 1) return i + (y + 2 >= ny ? 2 - ny : 2) * nx;
+    return i + (z + 2 >= nz ? 2 - nz : 2) * nx * ny;
+  }
+  __device__ __forceinline__ int m2(int a) const {
+    if (a == 0) return i + (x < 2 ? nx - 2 : -2);
+    if (a == 1) return i + (y < 2 ? ny - 2 : -2) * nx;
+    return i + (z < 2 ? nz - 2 : -2) * nx * ny;
+  }
+};
+
+// E at the site (central difference of phi plus the applied field)
 template <typename T>
-__device__ __forceinline__ void efield(const AdjK<T> &k, const T *phi, long long j, T E[3]) {
-  long long jp[3], jm[3];
-  nb6(k.d, j, jp, jm);
+__device__ __forceinline__ void efield(const AdjK<T> &k, const T *phi, const Nb32 &nb, T E[3]) {
 #pragma unroll
-  for (int a = 0; a < 3; ++a) E[a] = T(-0.5) * (phi[jp[a]] - phi[jm[a]]) + k.Eext[a];
+  for (int a = 0; a < 3; ++a) E[a] = T(-0.5) * (phi[nb.p(a)] - phi[nb.m(a)]) + k.Eext[a];
 }
-template <typename T> __device__ __forceinline__ T efield_a(const AdjK<T> &k, const T *phi, long long j, int a) {
-  long long jp[3], jm[3];
-  nb6(k.d, j, jp, jm);
-  return T(-0.5) * (phi[jp[a]] - phi[jm[a]]) + k.Eext[a];
+// component a of E at the axis neighbour i + a (up) or i - a
+template <typename T>
+__device__ __forceinline__ T efield_along(const AdjK<T> &k, const T *phi, const Nb32 &nb, int a, bool up) {
+  return up ? T(-0.5) * (phi[nb.p2(a)] - phi[nb.i]) + k.Eext[a] : T(-0.5) * (phi[nb.i] - phi[nb.m2(a)]) + k.Eext[a];
+}
+// E at the axis neighbour: along the axis from two sites away, across it from the face diagonals
+template <typename T>
+__device__ __forceinline__ void efield_beside(const AdjK<T> &k, const T *phi, const Nb32 &nb, int a, bool up, T E[3]) {
+  const int o = (up ? nb.p(a) : nb.m(a)) - nb.i;
+#pragma unroll
+  for (int b = 0; b < 3; ++b)
+    E[b] = b == a ? efield_along(k, phi, nb, a, up) : T(-0.5) * (phi[nb.p(b) + o] - phi[nb.m(b) + o]) + k.Eext[b];
 }
 
 __device__ __forceinline__ void block_partials(double v[kAdjPar], double *out) {
@@ -103,24 +148,22 @@ __device__ __forceinline__ void block_partials(double v[kAdjPar], double *out) {
 template <typename T, bool IONS>
 __global__ void __launch_bounds__(256, 2) ak_a(AdjK<T> k, AdjBufs<T> B, double *part) {
   const Dims d = k.d;
-  const long long N = d.N;
+  const int N = int(d.N);
   double acc[kAdjPar] = {0, 0, 0, 0};
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    int x, y, z;
-    coords(d, i, x, y, z);
-    long long nb[19];
-    neighbours19(d, x, y, z, nb);
-    const T rho[2] = {B.rho[i], B.rho[N + i]};
+  for (long long ii = blockIdx.x * (long long)blockDim.x + threadIdx.x; ii < N; ii += (long long)gridDim.x * blockDim.x) {
+    const int i = int(ii);
+    const Nb32 nb(d, i);
+    const T rho[2] = {B.rho[i], B.rho[size_t(N) + i]};
     const T rt = rho[0] + rho[1];
     const T inv_rho = rt > T(0) ? T(1) / rt : T(0);
-    const T J[3] = {B.J[i], B.J[N + i], B.J[2 * N + i]};
-    const T psi[2] = {B.psi[i], B.psi[N + i]};
+    const T J[3] = {B.J[i], B.J[size_t(N) + i], B.J[2 * size_t(N) + i]};
+    const T psi[2] = {B.psi[i], B.psi[size_t(N) + i]};
     // forward forces
     T S[2][3] = {{T(0), T(0), T(0)}, {T(0), T(0), T(0)}};
     if (k.G != T(0)) {
 #pragma unroll
       for (int q = 1; q < 19; ++q) {
-        const T pa = wq<T>(q) * B.psi[nb[q]], pb = wq<T>(q) * B.psi[N + nb[q]];
+        const T pa = wq<T>(q) * B.psi[nb[q]], pb = wq<T>(q) * B.psi[size_t(N) + nb[q]];
         S[0][0] += T(cx(q)) * pa; S[0][1] += T(cy(q)) * pa; S[0][2] += T(cz(q)) * pa;
         S[1][0] += T(cx(q)) * pb; S[1][1] += T(cy(q)) * pb; S[1][2] += T(cz(q)) * pb;
       }
@@ -132,8 +175,8 @@ __global__ void __launch_bounds__(256, 2) ak_a(AdjK<T> k, AdjBufs<T> B, double *
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         T Ep[3], Em[3];
-        efield(k, B.phi, nb[1 + 2 * a], Ep);
-        efield(k, B.phi, nb[2 + 2 * a], Em);
+        efield_beside(k, B.phi, nb, a, true, Ep);
+        efield_beside(k, B.phi, nb, a, false, Em);
         K[a] = (Ep[0] * Ep[0] + Ep[1] * Ep[1] + Ep[2] * Ep[2]) - (Em[0] * Em[0] + Em[1] * Em[1] + Em[2] * Em[2]);
         Fel[a] = de * K[a];
       }
@@ -142,10 +185,10 @@ __global__ void __launch_bounds__(256, 2) ak_a(AdjK<T> k, AdjBufs<T> B, double *
       const T inv_2D = T(0.5) / k.D;
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        const long long jm = nb[2 + 2 * a];
+        const int jm = nb.m(a);
         T tot = T(0);
 #pragma unroll
-        for (int s = 0; s < 2; ++s) tot += B.flux[(s * 3 + a) * N + i] + B.flux[(s * 3 + a) * N + jm];
+        for (int s = 0; s < 2; ++s) tot += B.flux[size_t(s * 3 + a) * N + i] + B.flux[size_t(s * 3 + a) * N + jm];
         Fel[a] += -tot * inv_2D;
       }
     }
@@ -200,20 +243,20 @@ __global__ void __launch_bounds__(256, 2) ak_a(AdjK<T> k, AdjBufs<T> B, double *
     }
     // Nernst-Planck advection and the physical velocity
     if (IONS) {
-      const T u[3] = {B.u[i], B.u[N + i], B.u[2 * N + i]};
+      const T u[3] = {B.u[i], B.u[size_t(N) + i], B.u[2 * size_t(N) + i]};
       T ub[3] = {T(0), T(0), T(0)};
 #pragma unroll
       for (int s = 0; s < 2; ++s) {
-        const T nbi = B.nbo[s * N + i], ni = B.n[s * N + i];
+        const T nbi = B.nbo[size_t(s) * N + i], ni = B.n[size_t(s) * N + i];
         T out = nbi;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-          const T nbp = B.nbo[s * N + nb[1 + 2 * a]], nbm = B.nbo[s * N + nb[2 + 2 * a]];
+          const T nbp = B.nbo[size_t(s) * N + nb.p(a)], nbm = B.nbo[size_t(s) * N + nb.m(a)];
           const T ua = u[a];
           out += (ua > T(0) ? ua * (nbp - nbi) : T(0)) + (ua < T(0) ? -ua * (nbm - nbi) : T(0));
           ub[a] += ni * (ua > T(0) ? (nbp - nbi) : (ua < T(0) ? (nbi - nbm) : T(0)));
         }
-        B.nbn[s * N + i] = out;
+        B.nbn[size_t(s) * N + i] = out;
       }
       const T phys[3] = {(J[0] + T(0.5) * (Phi[0][0] + Phi[1][0])) * inv_rho,
                          (J[1] + T(0.5) * (Phi[0][1] + Phi[1][1])) * inv_rho,
@@ -238,7 +281,7 @@ __global__ void __launch_bounds__(256, 2) ak_a(AdjK<T> k, AdjBufs<T> B, double *
       for (int a = 0; a < 3; ++a) {
         pf += Phib[s][a] * Fel[a];
         psc += Phib[s][a] * S[1 - s][a];
-        B.Sb[((1 - s) * 3 + a) * N + i] = -k.G * psi[s] * Phib[s][a];
+        B.Sb[size_t((1 - s) * 3 + a) * N + i] = -k.G * psi[s] * Phib[s][a];
       }
       rb[s] += pf * inv_rho;
       rtb -= pf * rho[s] * inv_rho * inv_rho;
@@ -249,15 +292,15 @@ __global__ void __launch_bounds__(256, 2) ak_a(AdjK<T> k, AdjBufs<T> B, double *
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       eb += T(0.25) * Felb[a] * K[a];
-      B.KC[a * N + i] = de * Felb[a];
-      B.Felb[a * N + i] = Felb[a];
-      B.Jb[a * N + i] = Jb[a];
+      B.KC[size_t(a) * N + i] = de * Felb[a];
+      B.Felb[size_t(a) * N + i] = Felb[a];
+      B.Jb[size_t(a) * N + i] = Jb[a];
     }
     B.epsb[i] = eb;
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
-      B.rb[s * N + i] = rb[s] + rtb;
-      B.psib[s * N + i] = psib[s];
+      B.rb[size_t(s) * N + i] = rb[s] + rtb;
+      B.psib[size_t(s) * N + i] = psib[s];
     }
   }
   block_partials(acc, part);
@@ -292,15 +335,13 @@ __global__ void __launch_bounds__(256) ak_b(AdjK<T> k, AdjBufs<T> B) {
 template <typename T, bool IONS>
 __global__ void __launch_bounds__(256, 2) ak_c(AdjK<T> k, AdjBufs<T> B, double *part) {
   const Dims d = k.d;
-  const long long N = d.N;
+  const int N = int(d.N);
   double acc[kAdjPar] = {0, 0, 0, 0};
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    int x, y, z;
-    coords(d, i, x, y, z);
-    long long nb[19];
-    neighbours19(d, x, y, z, nb);
+  for (long long ii = blockIdx.x * (long long)blockDim.x + threadIdx.x; ii < N; ii += (long long)gridDim.x * blockDim.x) {
+    const int i = int(ii);
+    const Nb32 nb(d, i);
     T E[3] = {T(0), T(0), T(0)};
-    if (k.field) efield(k, B.phi, i, E);
+    if (k.field) efield(k, B.phi, nb, E);
     T Eb[3] = {T(0), T(0), T(0)};
     if (IONS) {
       // ions through the face fluxes of faces (i, i+a) and (i-a, i)
@@ -308,8 +349,8 @@ __global__ void __launch_bounds__(256, 2) ak_c(AdjK<T> k, AdjBufs<T> B, double *
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         if (k.field) {
-          Efp[a] = T(0.5) * (E[a] + efield_a(k, B.phi, nb[1 + 2 * a], a));
-          Efm[a] = T(0.5) * (efield_a(k, B.phi, nb[2 + 2 * a], a) + E[a]);
+          Efp[a] = T(0.5) * (E[a] + efield_along(k, B.phi, nb, a, true));
+          Efm[a] = T(0.5) * (efield_along(k, B.phi, nb, a, false) + E[a]);
         } else {
           Efp[a] = Efm[a] = T(0);
         }
@@ -320,41 +361,41 @@ __global__ void __launch_bounds__(256, 2) ak_c(AdjK<T> k, AdjBufs<T> B, double *
         T add = T(0);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-          const T Fbp = B.Fb[(s * 3 + a) * N + i], Fbm = B.Fb[(s * 3 + a) * N + nb[2 + 2 * a]];
+          const T Fbp = B.Fb[size_t(s * 3 + a) * N + i], Fbm = B.Fb[size_t(s * 3 + a) * N + nb.m(a)];
           add += k.D * Fbp * (T(-1) - zs * T(0.5) * Efp[a]) + k.D * Fbm * (T(1) - zs * T(0.5) * Efm[a]);
         }
-        B.nbn[s * N + i] += add;
+        B.nbn[size_t(s) * N + i] += add;
       }
       if (k.field)
 #pragma unroll
-        for (int a = 0; a < 3; ++a) Eb[a] += T(0.5) * (B.Efb[a * N + i] + B.Efb[a * N + nb[2 + 2 * a]]);
+        for (int a = 0; a < 3; ++a) Eb[a] += T(0.5) * (B.Efb[size_t(a) * N + i] + B.Efb[size_t(a) * N + nb.m(a)]);
     }
     if (k.field) {
       // Kelvin: E_i enters Fel_{i-a,a} with + and Fel_{i+a,a} with -
       T kc = T(0);
 #pragma unroll
-      for (int a = 0; a < 3; ++a) kc += B.KC[a * N + nb[2 + 2 * a]] - B.KC[a * N + nb[1 + 2 * a]];
+      for (int a = 0; a < 3; ++a) kc += B.KC[size_t(a) * N + nb.m(a)] - B.KC[size_t(a) * N + nb.p(a)];
 #pragma unroll
       for (int b = 0; b < 3; ++b) Eb[b] += T(2) * E[b] * kc;
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        B.Eb[a * N + i] = Eb[a];
+        B.Eb[size_t(a) * N + i] = Eb[a];
         acc[a] += double(Eb[a]);
       }
     }
     // psi-bar: local part plus the transposed Shan-Chen sums, then rho-bar
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
-      T pb = B.psib[s * N + i];
+      T pb = B.psib[size_t(s) * N + i];
       if (k.G != T(0)) {
 #pragma unroll
         for (int q = 1; q < 19; ++q) {
-          const long long src = nb[opp(q)];  // i = src + c_q
-          pb += wq<T>(q) * (T(cx(q)) * B.Sb[(s * 3 + 0) * N + src] + T(cy(q)) * B.Sb[(s * 3 + 1) * N + src] +
-                            T(cz(q)) * B.Sb[(s * 3 + 2) * N + src]);
+          const int src = nb[opp(q)];  // i = src + c_q
+          pb += wq<T>(q) * (T(cx(q)) * B.Sb[size_t(s * 3 + 0) * N + src] + T(cy(q)) * B.Sb[size_t(s * 3 + 1) * N + src] +
+                            T(cz(q)) * B.Sb[size_t(s * 3 + 2) * N + src]);
         }
       }
-      B.rb[s * N + i] += pb * (T(1) - B.psi[s * N + i]);  // d psi / d rho = exp(-rho) = 1 - psi
+      B.rb[size_t(s) * N + i] += pb * (T(1) - B.psi[size_t(s) * N + i]);  // d psi / d rho = exp(-rho) = 1 - psi
     }
   }
   block_partials(acc, part);
@@ -377,20 +418,20 @@ template <typename T> __global__ void __launch_bounds__(256) ak_d(AdjK<T> k, Adj
 template <typename T, bool IONS>
 __global__ void __launch_bounds__(256) ak_e(AdjK<T> k, AdjBufs<T> B, double *part) {
   const Dims d = k.d;
-  const long long N = d.N;
+  const int N = int(d.N);
   double acc[kAdjPar] = {0, 0, 0, 0};
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    long long jp[3], jm[3];
-    nb6(d, i, jp, jm);
-    T rb[2] = {B.rb[i], B.rb[N + i]};
+  for (long long ii = blockIdx.x * (long long)blockDim.x + threadIdx.x; ii < N; ii += (long long)gridDim.x * blockDim.x) {
+    const int i = int(ii);
+    const Nb32 nb(d, i);
+    T rb[2] = {B.rb[i], B.rb[size_t(N) + i]};
     if (k.field) {
       const T li = B.lam[i], pi = B.phi[i], ei = B.eps[i];
       T eb = B.epsb[i];
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        const T lp = B.lam[jp[a]], lm = B.lam[jm[a]];
-        const T pp = B.phi[jp[a]], pm = B.phi[jm[a]];
-        const T kp = T(0.5) * (ei + B.eps[jp[a]]), km = T(0.5) * (B.eps[jm[a]] + ei);
+        const T lp = B.lam[nb.p(a)], lm = B.lam[nb.m(a)];
+        const T pp = B.phi[nb.p(a)], pm = B.phi[nb.m(a)];
+        const T kp = T(0.5) * (ei + B.eps[nb.p(a)]), km = T(0.5) * (B.eps[nb.m(a)] + ei);
         const T kbp = (li - lp) * (k.Eext[a] - pp + pi);
         const T kbm = (lm - li) * (k.Eext[a] - pi + pm);
         eb += T(0.5) * (kbp + kbm);
@@ -398,17 +439,17 @@ __global__ void __launch_bounds__(256) ak_e(AdjK<T> k, AdjBufs<T> B, double *par
       }
       if (IONS) {
         B.nbn[i] -= li;
-        B.nbn[N + i] += li;
+        B.nbn[size_t(N) + i] += li;
       }
       // eps = (eps_a (1 - c) + eps_b (1 + c))/2,  c = (rho_b - rho_a)/(rho_a + rho_b)
-      const T ra = B.rho[i], rbb = B.rho[N + i], rt = ra + rbb;
+      const T ra = B.rho[i], rbb = B.rho[size_t(N) + i], rt = ra + rbb;
       if (rt > T(0)) {
         const T dedc = T(0.5) * (k.eps_b - k.eps_a), ir2 = T(1) / (rt * rt);
         rb[0] += eb * dedc * (T(-2) * rbb * ir2);
         rb[1] += eb * dedc * (T(2) * ra * ir2);
       }
     }
-    const T Jb[3] = {B.Jb[i], B.Jb[N + i], B.Jb[2 * N + i]};
+    const T Jb[3] = {B.Jb[i], B.Jb[size_t(N) + i], B.Jb[2 * size_t(N) + i]};
 #pragma unroll
     for (int s = 0; s < 2; ++s)
 #pragma unroll
@@ -500,12 +541,12 @@ template <typename T> struct AdjLaunch {
     const AdjBufs<T> B = bufs(a);
     const long long N = c.d.N;
     if (c.nions) {
-      count_launch(), ak_a<T, true><<<kAdjBlocks, 256, 0, c.s>>>(k, B, part);
+      count_launch(), ak_a<T, true><<<kAdjGrid, 256, 0, c.s>>>(k, B, part);
       count_launch(), ak_b<T><<<grid_for(N, 256), 256, 0, c.s>>>(k, B);
-      count_launch(), ak_c<T, true><<<kAdjBlocks, 256, 0, c.s>>>(k, B, part);
+      count_launch(), ak_c<T, true><<<kAdjGrid, 256, 0, c.s>>>(k, B, part);
     } else {
-      count_launch(), ak_a<T, false><<<kAdjBlocks, 256, 0, c.s>>>(k, B, part);
-      count_launch(), ak_c<T, false><<<kAdjBlocks, 256, 0, c.s>>>(k, B, part);
+      count_launch(), ak_a<T, false><<<kAdjGrid, 256, 0, c.s>>>(k, B, part);
+      count_launch(), ak_c<T, false><<<kAdjGrid, 256, 0, c.s>>>(k, B, part);
     }
     if (c.has_field) count_launch(), ak_d<T><<<grid_for(N, 256), 256, 0, c.s>>>(k, B);
   }
@@ -513,9 +554,9 @@ template <typename T> struct AdjLaunch {
     const AdjK<T> k = make(c);
     const AdjBufs<T> B = bufs(a);
     if (c.nions)
-      count_launch(), ak_e<T, true><<<kAdjBlocks, 256, 0, c.s>>>(k, B, part);
+      count_launch(), ak_e<T, true><<<kAdjGridE, 256, 0, c.s>>>(k, B, part);
     else
-      count_launch(), ak_e<T, false><<<kAdjBlocks, 256, 0, c.s>>>(k, B, part);
+      count_launch(), ak_e<T, false><<<kAdjGridE, 256, 0, c.s>>>(k, B, part);
   }
   static void seed(const Ctx &c, const void *f, void *fb, const double mom[4], double scale) {
     const AdjK<T> k = make(c);

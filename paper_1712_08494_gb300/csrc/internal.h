@@ -143,6 +143,9 @@ int poisson_reset(Poisson *p, cudaStream_t s);  // new state: no previous soluti
 // Eager solve for c.phi from c.eps and c.q: returns the cycle count, -(count+2)
 // if the cap was reached before the tolerance, -1 on a CUDA error.
 int poisson_solve(Poisson *p, Ctx &c, double *relres);
+// The solve without a host wait, where it is one launch (its outcome goes to the
+// status word and the totals of poisson_read); 1 where it needs the host, -1 on error.
+int poisson_issue(Poisson *p, Ctx &c);
 // Records the solve into the graph being captured on c.s, its cycles under a
 // conditional WHILE node driven by `handle`.  Returns 0 or -1.
 int poisson_capture(Poisson *p, Ctx &c, cudaGraphConditionalHandle handle);
@@ -198,7 +201,10 @@ struct AdjArgs {
   void *rb, *Jb, *Felb, *KC, *Sb, *psib, *epsb, *Fb, *Efb, *Eb, *qadj;  // work arrays
   const void *lam;                                       // adjoint potential (compute type)
 };
-constexpr int kAdjBlocks = 1024;  // fixed grid of the passes with parameter sums
+constexpr int kAdjBlocks = 1024;  // partial sums of the passes with parameter sums
+// Their fixed grids: one resident wave of the 152 SMs (two blocks per SM at 128
+// registers, three at 80); 1024 blocks ran as 3.4 waves.
+constexpr int kAdjGrid = 304, kAdjGridE = 456;
 constexpr int kAdjPar = 4;        // dJ/dE_x, dJ/dE_y, dJ/dE_z, dJ/dG per block
 struct AdjOps {
   // passes before the adjoint Poisson solve (its right-hand side lands in qadj)

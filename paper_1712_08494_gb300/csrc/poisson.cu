@@ -772,6 +772,13 @@ int poisson_solve(Poisson *p, Ctx &c, double *relres) {
   return p->fp64 ? enqueue<double>(p, c, none, false, relres) : enqueue<float>(p, c, none, false, relres);
 }
 
+int poisson_issue(Poisson *p, Ctx &c) {
+  if (!p->spec && p->pgrid == 0) return 1;
+  double rr = 0.0;
+  cudaGraphConditionalHandle none = 0;
+  return p->fp64 ? enqueue<double>(p, c, none, true, &rr) : enqueue<float>(p, c, none, true, &rr);
+}
+
 int poisson_capture(Poisson *p, Ctx &c, cudaGraphConditionalHandle handle) {
   double rr = 0;
   return p->fp64 ? enqueue<double>(p, c, handle, true, &rr) : enqueue<float>(p, c, handle, true, &rr);
