@@ -210,9 +210,14 @@ __global__ void __launch_bounds__(256, 2) ak_a(AdjK<T> k, AdjBufs<T> B, double *
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
       const T usq = ue[s][0] * ue[s][0] + ue[s][1] * ue[s][1] + ue[s][2] * ue[s][2];
+      // all 19 loads before the first store: through the buffers' plain pointers
+      // a load may not pass a store, and one at a time each waits for memory
+      T fs[19];
+#pragma unroll
+      for (int q = 0; q < 19; ++q) fs[q] = B.fbo[(size_t)(s * 19 + q) * N + nb[q]];  // population sent to i + c_q
 #pragma unroll
       for (int q = 0; q < 19; ++q) {
-        const T fsb = B.fbo[(size_t)(s * 19 + q) * N + nb[q]];  // population sent to i + c_q
+        const T fsb = fs[q];
         B.fbn[(size_t)(s * 19 + q) * N + i] = keep * fsb;
         const T eb = fsb * itau;
         const T cu = T(cx(q)) * ue[s][0] + T(cy(q)) * ue[s][1] + T(cz(q)) * ue[s][2];
@@ -416,7 +421,7 @@ template <typename T> __global__ void __launch_bounds__(256) ak_d(AdjK<T> k, Adj
 
 // ------------------------------------------------------------------ ak_e
 template <typename T, bool IONS>
-__global__ void __launch_bounds__(256) ak_e(AdjK<T> k, AdjBufs<T> B, double *part) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) ak_e(AdjK<T> k, AdjBufs<T> B, double *part) {
   const Dims d = k.d;
   const int N = int(d.N);
   double acc[kAdjPar] = {0, 0, 0, 0};
@@ -451,12 +456,14 @@ __global__ void __launch_bounds__(256) ak_e(AdjK<T> k, AdjBufs<T> B, double *par
     }
     const T Jb[3] = {B.Jb[i], B.Jb[size_t(N) + i], B.Jb[2 * size_t(N) + i]};
 #pragma unroll
-    for (int s = 0; s < 2; ++s)
+    for (int s = 0; s < 2; ++s) {
+      T v[19];  // loads before stores, as in ak_a
 #pragma unroll
-      for (int q = 0; q < 19; ++q) {
-        const size_t o = (size_t)(s * 19 + q) * N + i;
-        B.fbn[o] += rb[s] + T(cx(q)) * Jb[0] + T(cy(q)) * Jb[1] + T(cz(q)) * Jb[2];
-      }
+      for (int q = 0; q < 19; ++q) v[q] = B.fbn[(size_t)(s * 19 + q) * N + i];
+#pragma unroll
+      for (int q = 0; q < 19; ++q)
+        B.fbn[(size_t)(s * 19 + q) * N + i] = v[q] + (rb[s] + T(cx(q)) * Jb[0] + T(cy(q)) * Jb[1] + T(cz(q)) * Jb[2]);
+    }
   }
   block_partials(acc, part);
 }

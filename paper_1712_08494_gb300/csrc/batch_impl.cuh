@@ -38,8 +38,17 @@ __global__ void __launch_bounds__(kPB, kPBlocks)
   unsigned cid;
   asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(cid));
   const int b = rec0 + int(cid);
-  const BatchRec<S, T> &B = recs[b];
-  const StepK<T> &k = B.k;
+  // the box's record in shared memory, its model constants by value: a barrier
+  // empties the L1, and stores through the fields' pointers would have each
+  // constant read again from memory
+  __shared__ BatchRec<S, T> B;
+  {
+    const int *src = reinterpret_cast<const int *>(recs + b);
+    int *dst = reinterpret_cast<int *>(&B);
+    for (int w = threadIdx.x; w < int(sizeof(B) / sizeof(int)); w += blockDim.x) dst[w] = src[w];
+  }
+  __syncthreads();
+  const StepK<T> k = B.k;
   const long long N = k.d.N;
   const long long r0 = tm.rank(), G = tm.size();
   int cur = par[2 * b], ncur = par[2 * b + 1];
