@@ -116,6 +116,13 @@ struct SphereBox {
     }
     tot = unsigned(cnt[0]) * unsigned(cnt[1]) * unsigned(cnt[2]);
   }
+  // w more nodes at both ends of every row
+  __device__ __forceinline__ void widen_x(int w) {
+    cnt[0] = min(n[0], cnt[0] + 2 * w);
+    lo[0] -= w % n[0];
+    if (lo[0] < 0) lo[0] += n[0];
+    tot = unsigned(cnt[0]) * unsigned(cnt[1]) * unsigned(cnt[2]);
+  }
   // coordinates of the t-th node (t < tot), wrapped into the box
   __device__ __forceinline__ void node(unsigned t, int &x, int &y, int &z) const {
     const unsigned r = t / unsigned(cnt[0]), oz = r / unsigned(cnt[1]);

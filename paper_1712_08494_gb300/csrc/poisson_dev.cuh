@@ -1139,21 +1139,39 @@ __device__ __forceinline__ void residual_quad(const PArgs<T> &a, const Level<T> 
   }
 }
 
+// The last five levels of a block's sum tree by one warp: the same pairs as the
+// shared-memory levels (t and t + w), without their barriers and round trips.
+template <int M, int STRIDE> __device__ __forceinline__ void warp_tail(double (&v)[M], double *sh) {
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int m = 0; m < M; ++m) v[m] = sh[m * STRIDE + threadIdx.x];
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1)
+#pragma unroll
+      for (int m = 0; m < M; ++m) v[m] += __shfl_down_sync(0xffffffffu, v[m], w);
+    if (threadIdx.x == 0)
+#pragma unroll
+      for (int m = 0; m < M; ++m) sh[m * STRIDE] = v[m];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int m = 0; m < M; ++m) v[m] = sh[m * STRIDE];
+  __syncthreads();
+}
+
 // Fixed-order sums of M values over the block at once: a shared-memory tree
 // whose levels add all M values behind one set of barriers.  sh: M kPB doubles.
 template <int M> __device__ __forceinline__ void block_sums(double (&v)[M], double *sh) {
 #pragma unroll
   for (int m = 0; m < M; ++m) sh[m * kPB + threadIdx.x] = v[m];
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+  for (int w = blockDim.x / 2; w >= 32; w >>= 1) {
     if (threadIdx.x < w)
 #pragma unroll
       for (int m = 0; m < M; ++m) sh[m * kPB + threadIdx.x] += sh[m * kPB + threadIdx.x + w];
     __syncthreads();
   }
-#pragma unroll
-  for (int m = 0; m < M; ++m) v[m] = sh[m * kPB];
-  __syncthreads();
+  warp_tail<M, kPB>(v, sh);
 }
 // the team's sums of M per-thread values, identical in every block; false on abort
 template <int M, class Team>

@@ -104,15 +104,13 @@ template <int M> __device__ __forceinline__ void block_sum_m(double (&v)[M], dou
 #pragma unroll
   for (int m = 0; m < M; ++m) sh[m * kSB + threadIdx.x] = v[m];
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+  for (int w = blockDim.x / 2; w >= 32; w >>= 1) {
     if (threadIdx.x < w)
 #pragma unroll
       for (int m = 0; m < M; ++m) sh[m * kSB + threadIdx.x] += sh[m * kSB + threadIdx.x + w];
     __syncthreads();
   }
-#pragma unroll
-  for (int m = 0; m < M; ++m) v[m] = sh[m * kSB];
-  __syncthreads();
+  warp_tail<M, kSB>(v, sh);
 }
 // The blocks' sums of M per-thread values into part[m nb + blockIdx.x], and
 // after the grid barrier the M grid sums, added by every block in the same

@@ -12,6 +12,8 @@
 //   k_np       finite-volume Nernst-Planck update, upwind advection        (II.B)
 #pragma once
 
+#include <type_traits>
+
 #include "internal.h"
 #include "dfloat.cuh"
 
@@ -440,10 +442,11 @@ __device__ __forceinline__ void collide_site(const StepK<T> &k, const S *__restr
 //
 // With colloids a site away from every sphere (near == 0) has solid fraction
 // zero and no solid neighbour, itself and its neighbours: it takes the code of
-// a box without colloids, which gives the same bits without the 18 mask bytes
-// per component and the divisions by solid fractions of one: 256^3 suspension
-// 1305 -> 938 us, coated 128^3 drop 401 -> 292.  FP64 keeps one path: its boxes
-// are small, most warps near a sphere would take both (32^3: 75 -> 103 us).
+// a box without colloids, without the 18 mask bytes per component and the
+// divisions by solid fractions of one; k_collide_near does the others.  Both
+// together: 256^3 suspension 1305 -> 858 us, coated 128^3 drop 401 -> 267.  FP64
+// keeps one form for all sites: it runs small boxes, where the second kernel's
+// few sites take longer than the box (32^3: 75 -> 125 us).
 template <typename S, typename T, int NC, bool SOL, bool IONS>
 __global__ void __launch_bounds__(256, NC == 1 ? 4 : 3)
     k_collide(StepK<T> k, const S *__restrict__ f, S *__restrict__ fn, const T *__restrict__ rhoF,
@@ -453,12 +456,34 @@ __global__ void __launch_bounds__(256, NC == 1 ? 4 : 3)
               const double *__restrict__ cv, T *__restrict__ u_out, T *__restrict__ flux_out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= int(k.d.N)) return;
-  if (SOL && (sizeof(T) == 8 || near[i]))
-    collide_site<S, T, NC, SOL, IONS, true>(k, f, fn, rhoF, JF, psiF, eps, phi, n, psi_f, solid, owner, cv, u_out,
+  constexpr bool kSplit = SOL && sizeof(T) == 4;
+  if (kSplit && near[i]) return;  // k_collide_near
+  collide_site<S, T, NC, SOL && !kSplit, IONS, true>(k, f, fn, rhoF, JF, psiF, eps, phi, n, psi_f, solid, owner, cv, u_out,
                                             flux_out, i);
-  else
-    collide_site<S, T, NC, false, IONS, true>(k, f, fn, rhoF, JF, psiF, eps, phi, n, psi_f, solid, owner, cv, u_out,
-                                              flux_out, i);
+}
+
+// The sites near a colloid, over the boxes around the spheres (up to 16 blocks
+// each): in k_collide their warps would run both forms, and both forms would
+// share its registers.  Where spheres' boxes overlap a site is done again with
+// the same result.
+template <typename S, typename T, int NC, bool IONS>
+__global__ void __launch_bounds__(256, 2)
+    k_collide_near(StepK<T> k, const S *__restrict__ f, S *__restrict__ fn, const T *__restrict__ rhoF,
+                   const T *__restrict__ JF, const T *__restrict__ psiF, const T *__restrict__ eps,
+                   const T *__restrict__ phi, const T *__restrict__ n, const T *__restrict__ psi_f,
+                   const uint8_t *__restrict__ solid, const uint8_t *__restrict__ near, const int *__restrict__ owner,
+                   const double *__restrict__ cv, T *__restrict__ u_out, T *__restrict__ flux_out,
+                   const double *__restrict__ cx, const double *__restrict__ cr, int slabs) {
+  const int j = blockIdx.x / slabs, sl = blockIdx.x - j * slabs;
+  const SphereBox box = block_box(k.d, cx + 3 * j, cr[j], 2.01);
+  for (unsigned t = unsigned(sl) * blockDim.x + threadIdx.x; t < box.tot; t += unsigned(slabs) * blockDim.x) {
+    int x, y, z;
+    box.node(t, x, y, z);
+    const int i = int(site(k.d, x, y, z));
+    if (near[i])
+      collide_site<S, T, NC, true, IONS, true>(k, f, fn, rhoF, JF, psiF, eps, phi, n, psi_f, solid, owner, cv, u_out,
+                                               flux_out, i);
+  }
 }
 
 // ---------------------------------------------------------------- k_np
@@ -518,14 +543,120 @@ __device__ __forceinline__ void np_site(const StepK<T> &k, const T *__restrict__
   }
 }
 
-template <typename T, bool SOL>
+// np_site on W consecutive sites of a row (W words fill 16 bytes, rows of a
+// multiple of W sites, no solid node or neighbour): 16-byte loads of the row
+// and of its neighbour rows and one word past each end, 35 loads for W sites
+// instead of 35 each; the same arithmetic per site.  The pass reads and writes
+// 52 B a site and was bound by its load instructions.
+template <typename T, int W> struct alignas(16) Words {
+  T v[W];
+};
+template <typename T, int W>
+__device__ __forceinline__ void np_row(const StepK<T> &k, const T *__restrict__ n, T *__restrict__ nn,
+                                       const T *__restrict__ flux, const T *__restrict__ u, const unsigned g) {
+  using V = Words<T, W>;
+  const unsigned nx = unsigned(k.d.nx), ny = unsigned(k.d.ny), nz = unsigned(k.d.nz), nxy = nx * ny;
+  const size_t N = size_t(k.d.N);
+  const unsigned i = g * W, r = i / nx, x = i - r * nx, z = r / ny, y = r - z * ny;
+  auto row = [](const T *p) { return *reinterpret_cast<const V *>(p); };
+  const unsigned xm = x == 0 ? i + nx - 1u : i - 1u, xp = x + W == nx ? i + W - nx : i + W;  // one word past each end
+  const unsigned jm[3] = {i, y == 0 ? i + (ny - 1u) * nx : i - nx, z == 0 ? i + (nz - 1u) * nxy : i - nxy};
+  const unsigned jp[3] = {i, y + 1u == ny ? i - (ny - 1u) * nx : i + nx, z + 1u == nz ? i - (nz - 1u) * nxy : i + nxy};
+  // values before and after each site along x from the row and the words past its ends
+  auto before = [](const V &v, T e) {
+    V o;
+#pragma unroll
+    for (int c = 0; c < W; ++c) o.v[c] = c ? v.v[c ? c - 1 : 0] : e;
+    return o;
+  };
+  auto after = [](const V &v, T e) {
+    V o;
+#pragma unroll
+    for (int c = 0; c < W; ++c) o.v[c] = c + 1 < W ? v.v[c + 1 < W ? c + 1 : c] : e;
+    return o;
+  };
+  V ui[3], um[3], up[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) ui[a] = row(u + a * N + i);
+  um[0] = before(ui[0], u[xm]);
+  up[0] = after(ui[0], u[xp]);
+#pragma unroll
+  for (int a = 1; a < 3; ++a) {
+    um[a] = row(u + a * N + jm[a]);
+    up[a] = row(u + a * N + jp[a]);
+  }
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const T *ns = n + s * N;
+    const V ni = row(ns + i);
+    V nm[3], np[3], fi[3], fm[3];
+    nm[0] = before(ni, ns[xm]);
+    np[0] = after(ni, ns[xp]);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) fi[a] = row(flux + (s * 3 + a) * N + i);
+    fm[0] = before(fi[0], flux[s * 3 * N + xm]);
+#pragma unroll
+    for (int a = 1; a < 3; ++a) {
+      nm[a] = row(ns + jm[a]);
+      np[a] = row(ns + jp[a]);
+      fm[a] = row(flux + (s * 3 + a) * N + jm[a]);
+    }
+    V o;
+#pragma unroll
+    for (int c = 0; c < W; ++c) {
+      T div = T(0);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) div += fi[a].v[c] - fm[a].v[c];
+      T out = T(0), in = T(0);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        out += fmax(ui[a].v[c], T(0)) * ni.v[c];
+        out += fmax(-ui[a].v[c], T(0)) * ni.v[c];
+      }
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        in += fmax(um[a].v[c], T(0)) * nm[a].v[c];
+        in += fmax(-up[a].v[c], T(0)) * np[a].v[c];
+      }
+      o.v[c] = ((ni.v[c] + div) - out) + in;
+    }
+    *reinterpret_cast<V *>(nn + s * N + i) = o;
+  }
+}
+
+// A thread takes W sites of a row; groups with a site near a colloid are left
+// to k_np_near.
+template <typename T, int W>
+__device__ __forceinline__ bool near_group(const uint8_t *__restrict__ near, size_t g) {
+  using M = typename std::conditional<W == 4, unsigned, typename std::conditional<W == 2, unsigned short, uint8_t>::type>::type;
+  return reinterpret_cast<const M *>(near)[g] != 0;
+}
+template <typename T, bool SOL, int W>
 __global__ void __launch_bounds__(256) k_np(StepK<T> k, const T *__restrict__ n, T *__restrict__ nn,
                                             const T *__restrict__ flux, const T *__restrict__ u,
                                             const uint8_t *__restrict__ solid, const uint8_t *__restrict__ near) {
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= k.d.N) return;
-  if (SOL && (sizeof(T) == 8 || near[i])) np_site<T, SOL>(k, n, nn, flux, u, solid, i);
-  else np_site<T, false>(k, n, nn, flux, u, solid, i);
+  const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (g * W >= k.d.N) return;
+  constexpr bool kSplit = SOL && sizeof(T) == 4;  // as k_collide
+  if (kSplit && near_group<T, W>(near, size_t(g))) return;
+  if constexpr (W > 1) np_row<T, W>(k, n, nn, flux, u, unsigned(g));
+  else np_site<T, SOL && !kSplit>(k, n, nn, flux, u, solid, g);
+}
+template <typename T, int W>
+__global__ void __launch_bounds__(256) k_np_near(StepK<T> k, const T *__restrict__ n, T *__restrict__ nn,
+                                                 const T *__restrict__ flux, const T *__restrict__ u,
+                                                 const uint8_t *__restrict__ solid, const uint8_t *__restrict__ near,
+                                                 const double *__restrict__ cx, const double *__restrict__ cr,
+                                                 int slabs) {
+  const int j = blockIdx.x / slabs, sl = blockIdx.x - j * slabs;
+  SphereBox box = block_box(k.d, cx + 3 * j, cr[j], 2.01);
+  box.widen_x(W - 1);  // the rest of the groups at the ends
+  for (unsigned t = unsigned(sl) * blockDim.x + threadIdx.x; t < box.tot; t += unsigned(slabs) * blockDim.x) {
+    int x, y, z;
+    box.node(t, x, y, z);
+    const size_t i = size_t(site(k.d, x, y, z));
+    if (near_group<T, W>(near, i / W)) np_site<T, true>(k, n, nn, flux, u, solid, (long long)i);
+  }
 }
 
 // ---------------------------------------------------------------- init / read-out
@@ -1114,6 +1245,12 @@ template <typename S, typename T> struct Launch {
         k, (const S *)c.f[c.cur], (S *)c.f[1 - c.cur], (const T *)c.rho, (const T *)c.J, (const T *)c.psi,
         (const T *)c.eps, (const T *)c.phit, (const T *)c.n[c.ncur], (const T *)c.psi_f, c.solid, c.near,
         c.owner, c.cv, (T *)c.u, (T *)c.flux);
+    if (!SOL || sizeof(T) == 8) return;
+    const int sl = colloid_slabs(c.ncoll);
+    count_launch(), k_collide_near<S, T, NC, IONS><<<c.ncoll * sl, B, 0, c.s>>>(
+        k, (const S *)c.f[c.cur], (S *)c.f[1 - c.cur], (const T *)c.rho, (const T *)c.J, (const T *)c.psi,
+        (const T *)c.eps, (const T *)c.phit, (const T *)c.n[c.ncur], (const T *)c.psi_f, c.solid, c.near,
+        c.owner, c.cv, (T *)c.u, (T *)c.flux, c.cx, c.cr, sl);
   }
   static void collide(Ctx &c) {
     const bool ions = c.nions > 0;
@@ -1130,10 +1267,20 @@ template <typename S, typename T> struct Launch {
     auto k = make_stepk<T>(c);
     const T *n = (const T *)c.n[c.ncur];
     T *nn = (T *)c.n[1 - c.ncur];
-    if (c.solids)
-      count_launch(), k_np<T, true><<<grid_for(c.d.N, B), B, 0, c.s>>>(k, n, nn, (const T *)c.flux, (const T *)c.u, c.solid, c.near);
-    else
-      count_launch(), k_np<T, false><<<grid_for(c.d.N, B), B, 0, c.s>>>(k, n, nn, (const T *)c.flux, (const T *)c.u, c.solid, c.near);
+    // FP64 goes site by site: it is bound by the FP64 rate, and its boxes are
+    // small (32^3: 10 us, by pairs 18)
+    constexpr int W = sizeof(T) == 4 ? 4 : 1;
+    const bool wide = c.d.nx % W == 0;
+    if (c.solids) wide ? np_launch<true, W>(c, k, n, nn) : np_launch<true, 1>(c, k, n, nn);
+    else wide ? np_launch<false, W>(c, k, n, nn) : np_launch<false, 1>(c, k, n, nn);
+  }
+  template <bool SOL, int W> static void np_launch(Ctx &c, const StepK<T> &k, const T *n, T *nn) {
+    count_launch(), k_np<T, SOL, W><<<grid_for(c.d.N / W, B), B, 0, c.s>>>(k, n, nn, (const T *)c.flux, (const T *)c.u,
+                                                                           c.solid, c.near);
+    if (!SOL || sizeof(T) == 8) return;
+    const int sl = colloid_slabs(c.ncoll);
+    count_launch(), k_np_near<T, W><<<c.ncoll * sl, B, 0, c.s>>>(k, n, nn, (const T *)c.flux, (const T *)c.u, c.solid,
+                                                                 c.near, c.cx, c.cr, sl);
   }
   // one resident wave of k_obs (at most max_blocks); returns its block count
   template <int NC> static int obs_launch(Ctx &c, double *partials, int max_blocks) {
