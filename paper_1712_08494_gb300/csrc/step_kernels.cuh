@@ -416,7 +416,11 @@ __device__ __forceinline__ void collide_site(const StepK<T> &k, const S *__restr
     const T usq = ue[s][0] * ue[s][0] + ue[s][1] * ue[s][1] + ue[s][2] * ue[s][2];
 #pragma unroll
     for (int qd = 0; qd < 19; ++qd) {
-      const T cu = T(cx(qd)) * ue[s][0] + T(cy(qd)) * ue[s][1] + T(cz(qd)) * ue[s][2];
+      // c . u_e without the products by zero, which the compiler has to keep
+      T cu = T(0);
+      if (cx(qd)) cu = T(cx(qd)) * ue[s][0];
+      if (cy(qd)) cu = cx(qd) ? cu + T(cy(qd)) * ue[s][1] : T(cy(qd)) * ue[s][1];
+      if (cz(qd)) cu = cx(qd) || cy(qd) ? cu + T(cz(qd)) * ue[s][2] : T(cz(qd)) * ue[s][2];
       const T feq = wq<T>(qd) * rho[s] * (T(1) + T(3) * cu + T(4.5) * cu * cu - T(1.5) * usq);
       const T fpost = fl[qd] + (feq - fl[qd]) * k.inv_tau;
       if (qd == 0) {
