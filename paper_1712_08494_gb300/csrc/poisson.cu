@@ -544,7 +544,7 @@ Poisson *poisson_create(const Ctx &c, int fp64) {
     }
     p->dev = alloc<PDev>(p, 1);
     p->bar = alloc<Bar>(p, 1);
-    p->part = alloc<double>(p, 3 * spectral_grid(p->spec) + 8);
+    p->part = alloc<double>(p, part_doubles(spectral_grid(p->spec)));
     if ((fp64 ? !p->phi_prev : (!p->prev_hi || !p->prev_lo)) || !p->dev || !p->bar || !p->part) {
       poisson_destroy(p);
       return nullptr;
@@ -571,7 +571,8 @@ Poisson *poisson_create(const Ctx &c, int fp64) {
     else
       persistent_setup<float, true>(p, c);
   }
-  p->part = alloc<double>(p, 3 * std::max(p->nred, p->pgrid) + 8);
+  // partials of the multi-kernel path (nred blocks), of one team or of one cluster (at most 16 blocks)
+  p->part = alloc<double>(p, part_doubles(std::max({p->nred, p->pgrid, 16})));
   if (!ok || (fp64 ? !p->phi_prev : (!p->prev_hi || !p->prev_lo)) || !p->part || !p->dev) {
     poisson_destroy(p);
     return nullptr;

@@ -10,6 +10,7 @@
 
 #include "internal.h"
 #include "dfloat.cuh"
+#include "team_part.h"
 
 namespace lbeh {
 
@@ -996,6 +997,7 @@ struct GridTeam {
 
 struct ClusterTeam {
   unsigned crank, csize;
+  mutable unsigned long long gen = 0;  // barriers passed in this launch
   __device__ ClusterTeam() {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(csize));
@@ -1005,6 +1007,7 @@ struct ClusterTeam {
   __device__ int block() const { return int(crank); }
   __device__ int nblocks() const { return int(csize); }
   __device__ bool sync() const {
+    ++gen;
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
     return true;
   }
@@ -1021,7 +1024,7 @@ template <typename T> struct PArgs {
   double ex, ey, ez;
   PDev *st;
   int *status;
-  double *part;  // [3][blocks of the team]
+  double *part;  // block sums of two reductions in turn (team_part.h)
   Bar *bar;
   long long spin_limit;  // polls of a grid-barrier wait before time-out (cooperative solve)
 };
@@ -1184,13 +1187,13 @@ __device__ __forceinline__ bool team_sums(double (&v)[M], double *part, const Te
   const int nb = tm.nblocks();
   if (threadIdx.x == 0)
 #pragma unroll
-    for (int m = 0; m < M; ++m) part[m * nb + tm.block()] = v[m];
+    for (int m = 0; m < M; ++m) part[part_at(tm.gen, m, nb, tm.block())] = v[m];
   if (!tm.sync()) return false;
 #pragma unroll
   for (int m = 0; m < M; ++m) v[m] = 0.0;
   for (int b = threadIdx.x; b < nb; b += blockDim.x)
 #pragma unroll
-    for (int m = 0; m < M; ++m) v[m] += part[m * nb + b];
+    for (int m = 0; m < M; ++m) v[m] += part[part_at(tm.gen - 1, m, nb, b)];
   block_sums<M>(v, sh);
   return true;
 }

@@ -112,15 +112,16 @@ template <int M> __device__ __forceinline__ void block_sum_m(double (&v)[M], dou
   }
   warp_tail<M, kSB>(v, sh);
 }
-// The blocks' sums of M per-thread values into part[m nb + blockIdx.x], and
-// after the grid barrier the M grid sums, added by every block in the same
-// fixed order (every block holds bitwise the same scalars and takes the same
-// branches).
-template <int M> __device__ __forceinline__ void put_block_sums(double (&v)[M], double *part, int nb, double *sh) {
+// The blocks' sums of M per-thread values into part, and after the grid barrier
+// (the next one that the block passes) the M grid sums, added by every block in
+// the same fixed order (every block holds bitwise the same scalars and takes
+// the same branches).
+template <int M>
+__device__ __forceinline__ void put_block_sums(const GridTeam &tm, double (&v)[M], double *part, int nb, double *sh) {
   block_sum_m<M>(v, sh);
   if (threadIdx.x == 0)
 #pragma unroll
-    for (int m = 0; m < M; ++m) part[m * nb + blockIdx.x] = v[m];
+    for (int m = 0; m < M; ++m) part[part_at(tm.gen, m, nb, tm.block())] = v[m];
 }
 template <int M>
 __device__ __forceinline__ bool sync_sums(const GridTeam &tm, double *part, int nb, double (&v)[M], double *sh) {
@@ -129,7 +130,7 @@ __device__ __forceinline__ bool sync_sums(const GridTeam &tm, double *part, int 
   for (int m = 0; m < M; ++m) v[m] = 0.0;
   for (int b = threadIdx.x; b < nb; b += blockDim.x)
 #pragma unroll
-    for (int m = 0; m < M; ++m) v[m] += part[m * nb + b];
+    for (int m = 0; m < M; ++m) v[m] += part[part_at(tm.gen - 1, m, nb, b)];
   block_sum_m<M>(v, sh);
   return true;
 }
@@ -1282,7 +1283,7 @@ __global__ void __launch_bounds__(kSB, 2) k_spectral(SArgs<T> a) {
   }
   {
     double v[1] = {sq.get()};
-    put_block_sums<1>(v, pa.part, nb, sh);
+    put_block_sums<1>(tm, v, pa.part, nb, sh);
   }
   double qs[1];
   if (!sync_sums<1>(tm, pa.part, nb, qs, sh)) return;
@@ -1301,7 +1302,7 @@ __global__ void __launch_bounds__(kSB, 2) k_spectral(SArgs<T> a) {
     {
       double v[3];
       residual_cells<BIG, T, DFM>(a, qbar, qbar_df, sh, v[0], v[1], v[2]);
-      put_block_sums<3>(v, pa.part, nb, sh);
+      put_block_sums<3>(tm, v, pa.part, nb, sh);
       if (!sync_sums<3>(tm, pa.part, nb, v, sh)) return;
       r2 = v[0];
       b2 = v[1];
@@ -1332,7 +1333,7 @@ __global__ void __launch_bounds__(kSB, 2) k_spectral(SArgs<T> a) {
         update_cells<BIG, T>(a, al, he, sr, se);
         have_e = true;
         double v[2] = {sr.get(), se.get()};
-        put_block_sums<2>(v, pa.part, nb, sh);
+        put_block_sums<2>(tm, v, pa.part, nb, sh);
         if (!sync_sums<2>(tm, pa.part, nb, v, sh)) return;
         r2 = v[0];
         sum_e = v[1];
@@ -1376,7 +1377,7 @@ __global__ void __launch_bounds__(kSB, 2) k_spectral(SArgs<T> a) {
         tile_pass<MIX, BIG, T>(a, sm, 0, kInv, lw, StoreRZ<T>{a.w, a.r, &srz});
       }
       double rz[3] = {srz.get(), sr.get(), se.get()};
-      put_block_sums<3>(rz, pa.part, nb, sh);
+      put_block_sums<3>(tm, rz, pa.part, nb, sh);
       if (!sync_sums<3>(tm, pa.part, nb, rz, sh)) return;
       const double rho = rz[0];
       if (upd) {
@@ -1395,7 +1396,7 @@ __global__ void __launch_bounds__(kSB, 2) k_spectral(SArgs<T> a) {
         constexpr int W = 16 / sizeof(T);
         if (BIG && d.nx % W == 0) matvec_rows<T, W>(a, a.w, T(beta), first, v[0], v[1], v[2]);
         else matvec_update<T, DFM>(a, a.w, T(beta), first, sh, v[0], v[1], v[2]);
-        put_block_sums<3>(v, pa.part, nb, sh);
+        put_block_sums<3>(tm, v, pa.part, nb, sh);
       }
       double fs[3];
       if (!sync_sums<3>(tm, pa.part, nb, fs, sh)) return;
