@@ -223,6 +223,22 @@ bool stage_out(lbeh_handle *h, const double *dsrc, void *dst, int on_device, lon
                                  h->c.s));
 }
 
+// Whether a kernel can store elements of `elem` bytes at a caller's device
+// pointer.  FP64 buffers may lie wherever a copy reaches (any alignment, memory
+// of another GPU without peer access): those are copied from a staging buffer.
+// FP32 buffers have to be memory that kernels of this GPU can write.
+bool stores_reach(const void *p, size_t elem) {
+  if (reinterpret_cast<uintptr_t>(p) % elem) return false;
+  if (elem == 4) return true;
+  cudaPointerAttributes a{};
+  int dev = 0;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev);
+}
+
 // FP64 device copy of a compute-type field.
 const double *as_f64(lbeh_handle *h, const void *src, long long count, std::vector<void *> &tmp) {
   if (h->c.prec == LBEH_FP64) return (const double *)src;
@@ -1281,7 +1297,7 @@ int lbeh_step_adjoint(lbeh_handle *h, int nsteps, int ckpt_every, const lbeh_obs
     }
   }
   if (f0_user) {
-    if (out_dev && c.prec != LBEH_FP64) {
+    if (out_dev && c.prec != LBEH_FP64 && stores_reach(f0_user, 8)) {
       count_launch(), k_cvt<float, double><<<grid_for(38 * N, 256), 256, 0, c.s>>>((const float *)fb[cur], f0_user, 38 * N);
     } else {
       const double *f0 = as_f64(h, fb[cur], 38 * N, tmp);
@@ -1310,14 +1326,20 @@ int lbeh_get_fields(lbeh_handle *h, lbeh_fields *out) {
   const int f32 = out->dtype == LBEH_F32;
   const size_t e = f32 ? 4 : 8;
   // each wanted field goes straight to the caller's device buffer, or to a
-  // staging buffer of its element type and from there to the host
+  // staging buffer of its element type and from there to the caller's
   void *user[6] = {out->rho[0], c.ncomp == 2 ? out->rho[1] : nullptr, c.nions ? out->n[0] : nullptr,
                    c.nions ? out->n[1] : nullptr, out->phi, out->u};
   void *dev[6];
   bool any = false;
+  auto target = [&](void *p, size_t bytes) {
+    return out->on_device && stores_reach(p, e) ? p : stage_buf(h, bytes, tmp);
+  };
+  auto deliver = [&](void *p, const void *d, size_t bytes) {
+    if (p != d)
+      ok &= cuda_ok(cudaMemcpyAsync(p, d, bytes, out->on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c.s));
+  };
   for (int k = 0; k < 6; ++k) {
-    dev[k] = user[k];
-    if (user[k] && !out->on_device) dev[k] = stage_buf(h, e * (k == 5 ? 3 : 1) * N, tmp);
+    dev[k] = user[k] ? target(user[k], e * (k == 5 ? 3 : 1) * N) : nullptr;
     if (user[k] && !dev[k]) {
       free_tmp(h, tmp);
       return LBEH_ERR_OOM;
@@ -1325,19 +1347,17 @@ int lbeh_get_fields(lbeh_handle *h, lbeh_fields *out) {
     any |= user[k] != nullptr;
   }
   if (any) h->ops.read(c, dev, f32);
-  if (!out->on_device)
-    for (int k = 0; k < 6; ++k)
-      if (user[k])
-        ok &= cuda_ok(cudaMemcpyAsync(user[k], dev[k], e * (k == 5 ? 3 : 1) * N, cudaMemcpyDeviceToHost, c.s));
+  for (int k = 0; k < 6; ++k)
+    if (user[k]) deliver(user[k], dev[k], e * (k == 5 ? 3 : 1) * N);
   if (out->f) {
     const size_t bytes = e * c.ncomp * 19 * (size_t)N;
-    void *fd = out->on_device ? out->f : stage_buf(h, bytes, tmp);
+    void *fd = target(out->f, bytes);
     if (!fd) {
       free_tmp(h, tmp);
       return LBEH_ERR_OOM;
     }
     h->ops.get_f(c, fd, f32);
-    if (!out->on_device) ok &= cuda_ok(cudaMemcpyAsync(out->f, fd, bytes, cudaMemcpyDeviceToHost, c.s));
+    deliver(out->f, fd, bytes);
   }
   const int nc = c.ncoll;
   if (nc && (out->cx || out->cv || out->cf)) {
