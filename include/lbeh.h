@@ -265,7 +265,10 @@ int lbeh_observables_noalloc(int nx, int ny, int nz, int ncomp, int nions, int d
  * on_device.  Synchronises.  Afterwards the handle is in the state lbeh_step
  * would leave (fields of the last step included).  A Poisson solve of either
  * sweep that misses its tolerance returns LBEH_ERR_POISSON_NOT_CONVERGED with
- * the gradients filled in. */
+ * the gradients filled in.  A solve that runs out of its wait limit, or a
+ * non-finite value in the forward sweep, ends the call with
+ * LBEH_ERR_BARRIER_TIMEOUT or LBEH_ERR_NONFINITE and without gradients: the
+ * sweep goes at most one step beyond the one in which it happened. */
 typedef struct lbeh_obs_seed {
   double d_deformation; /* dJ/dD of the final state */
   const double *f_bar;  /* optional [2][19][N]: dJ/df(t_end) */

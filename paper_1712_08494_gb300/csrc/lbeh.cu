@@ -72,6 +72,7 @@ struct lbeh_handle {
   long long wait_limit = 0;     // barrier-wait polls of the Poisson solves (0: default)
   void *adj_block = nullptr;    // device memory of the adjoint calls, kept between them up to kAdjKeep
   size_t adj_block_bytes = 0;
+  int *watch = nullptr;         // pinned: status words of the last two steps of a sweep (StatusWatch)
 };
 
 std::atomic<long long> lbeh::g_launches{0};
@@ -716,6 +717,7 @@ static void destroy_handle(lbeh_handle *h) {
   poisson_destroy(h->pois);
   poisson_destroy(h->adj_pois);
   if (h->adj_block) cudaFree(h->adj_block);
+  if (h->watch) cudaFreeHost(h->watch);
   for (void *a : h->allocs) cudaFree(a);
   for (auto &b : h->stage) cudaFree(b.p);
   delete h;
@@ -1018,6 +1020,44 @@ struct DevArena {
     return p;
   }
 };
+
+// Status bits of a sweep's steps, read one step behind: next() copies the word
+// behind the work issued so far and waits for the copy of the call before, so
+// the device has the step just issued to run meanwhile.  A solve that gave up
+// waiting is then followed by one more at most; without the read each later
+// step of the sweep waited its own full limit.  At 96^3 and 20 steps the read
+// costs nothing that shows (29.33 ms with and without; 29.62 with the copy on
+// the sweep's own stream); a wait for each step's own word in both sweeps took
+// 29.08 to 29.90 ms.
+struct StatusWatch {
+  int *host = nullptr;
+  cudaStream_t s, cs;  // the sweep's stream, and the copy stream (the word's bits are only ever set)
+  cudaEvent_t issued = nullptr, ev[2] = {nullptr, nullptr};
+  int n = 0;
+  bool ok = true;
+  explicit StatusWatch(lbeh_handle *h) : s(h->c.s), cs(h->cs ? h->cs : h->c.s) {
+    if (!h->watch) ok = cuda_ok(cudaMallocHost(&h->watch, 2 * sizeof(int)));
+    if (!ok) h->watch = nullptr;
+    host = h->watch;
+    for (cudaEvent_t *e : {&issued, &ev[0], &ev[1]}) ok &= cuda_ok(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+  }
+  ~StatusWatch() {
+    for (cudaEvent_t e : {issued, ev[0], ev[1]})
+      if (e) cudaEventDestroy(e);
+  }
+  StatusWatch(const StatusWatch &) = delete;
+  StatusWatch &operator=(const StatusWatch &) = delete;
+  // bits of the step before (0 for the first); -1 on a CUDA error
+  int next(const int *word) {
+    const int k = n++ & 1;
+    if (!cuda_ok(cudaEventRecord(issued, s)) || !cuda_ok(cudaStreamWaitEvent(cs, issued, 0)) ||
+        !cuda_ok(cudaMemcpyAsync(host + k, word, sizeof(int), cudaMemcpyDeviceToHost, cs)) ||
+        !cuda_ok(cudaEventRecord(ev[k], cs)))
+      return -1;
+    if (n == 1) return 0;
+    return cuda_ok(cudaEventSynchronize(ev[k ^ 1])) ? host[k ^ 1] : -1;
+  }
+};
 }  // namespace
 
 int lbeh_step_adjoint(lbeh_handle *h, int nsteps, int ckpt_every, const lbeh_obs_seed *seed, lbeh_grads *out) {
@@ -1118,6 +1158,8 @@ int lbeh_step_adjoint(lbeh_handle *h, int nsteps, int ckpt_every, const lbeh_obs
     for (auto &x : ev) cudaEventDestroy(x);
     return rc;
   };
+  StatusWatch fwatch(h), rwatch(h);
+  if (!fwatch.ok || !rwatch.ok) return finish(cuda_fail(h, "adjoint setup"));
 
   // forward sweep: checkpoints of (f, n) every K steps, the potential of every step
   cudaEventRecord(ev[0], c.s);
@@ -1128,8 +1170,15 @@ int lbeh_step_adjoint(lbeh_handle *h, int nsteps, int ckpt_every, const lbeh_obs
       cudaMemcpyAsync(dst, c.f[c.cur], popB, cudaMemcpyDeviceToDevice, c.s);
       if (ionB) cudaMemcpyAsync(dst + popB, c.n[c.ncur], ionB, cudaMemcpyDeviceToDevice, c.s);
     }
-    const int rc = issue_steps(h, 1);  // no host wait between the steps
+    const int rc = issue_steps(h, 1);  // no host wait for this step
     if (rc != LBEH_OK) return finish(rc);
+    if (h->pois) {
+      const int bits = fwatch.next(c.status);
+      if (bits < 0) return finish(cuda_fail(h, "adjoint forward sweep"));
+      if ((bits & (ST_TIMEOUT | ST_NONFINITE)) ||
+          (h->status != LBEH_OK && h->status != LBEH_ERR_POISSON_NOT_CONVERGED))
+        return finish(finish_steps(h));
+    }
     cudaMemcpyAsync(phis + (size_t)t * phiB, c.phit, phiB, cudaMemcpyDeviceToDevice, c.s);
   }
   cudaEventRecord(ev[1], c.s);
@@ -1176,7 +1225,7 @@ int lbeh_step_adjoint(lbeh_handle *h, int nsteps, int ckpt_every, const lbeh_obs
   // reverse sweep, segment by segment from the last
   int cur = 0;
   long long cycles = 0;
-  // one-launch solves run without a host wait; their outcome is read at the end
+  // one-launch solves run without a host wait for their own outcome, which is read at the end
   const bool async = c.has_field && !poisson_needs_conditional(h->adj_pois);
   PoissonStats before{};
   if (async && poisson_read(h->adj_pois, c.s, &before) != 0) return finish(cuda_fail(h, "adjoint Poisson read-back"));
@@ -1194,7 +1243,8 @@ int lbeh_step_adjoint(lbeh_handle *h, int nsteps, int ckpt_every, const lbeh_obs
     if (c.prec == LBEH_FP64) cc.phi = (double *)cc.phit;
     return cc;
   };
-  for (int sg = nseg - 1; sg >= 0; --sg) {
+  bool gave_up = false;  // a solve of the reverse sweep ran out of its wait limit
+  for (int sg = nseg - 1; sg >= 0 && !gave_up; --sg) {
     const int ts = sg * K, L = std::min(nsteps, ts + K) - ts;
     cudaMemcpyAsync(seg, ck + (size_t)sg * stB, stB, cudaMemcpyDeviceToDevice, c.s);
     for (int j = 0; j + 1 < L; ++j) {
@@ -1203,7 +1253,7 @@ int lbeh_step_adjoint(lbeh_handle *h, int nsteps, int ckpt_every, const lbeh_obs
       h->ops.collide(cc);
       if (ionB) h->ops.np(cc);
     }
-    for (int j = L - 1; j >= 0; --j) {
+    for (int j = L - 1; j >= 0 && !gave_up; --j) {
       Ctx cc = step_ctx(ts + j, j);
       h->ops.macro(cc);
       h->ops.collide(cc);  // fields of the step: rho, J, psi, eps, q, u, face fluxes
@@ -1236,6 +1286,9 @@ int lbeh_step_adjoint(lbeh_handle *h, int nsteps, int ckpt_every, const lbeh_obs
       A.before_solve(cc, a, part);
       if (c.has_field && async) {
         if (poisson_issue(h->adj_pois, ca) != 0) return finish(cuda_fail(h, "adjoint Poisson solve"));
+        const int bits = rwatch.next(astatus);
+        if (bits < 0) return finish(cuda_fail(h, "adjoint Poisson solve"));
+        gave_up = (bits & ST_TIMEOUT) != 0;
       } else if (c.has_field) {
         double rr = 0.0;
         const int it = poisson_solve(h->adj_pois, ca, &rr);
