@@ -290,6 +290,18 @@ void free_tmp(lbeh_handle *h, std::vector<void *> &tmp, bool wait = true) {
   tmp.clear();
 }
 
+// Staging buffers of one call, returned to the pool on every way out of it.
+struct Staged {
+  lbeh_handle *h;
+  std::vector<void *> bufs;
+  explicit Staged(lbeh_handle *hh) : h(hh) {}
+  ~Staged() {
+    if (!bufs.empty()) free_tmp(h, bufs);
+  }
+  Staged(const Staged &) = delete;
+  Staged &operator=(const Staged &) = delete;
+};
+
 int check_params(const lbeh_params *p) {
   if (!p) return LBEH_ERR_INVALID_ARG;
   if (p->nx < 2 || p->ny < 2 || p->nz < 2) return LBEH_ERR_INVALID_ARG;
@@ -1158,6 +1170,8 @@ int lbeh_step_adjoint(lbeh_handle *h, int nsteps, int ckpt_every, const lbeh_obs
     for (auto &x : ev) cudaEventDestroy(x);
     return rc;
   };
+  Staged staged(h);
+  std::vector<void *> &tmp = staged.bufs;
   StatusWatch fwatch(h), rwatch(h);
   if (!fwatch.ok || !rwatch.ok) return finish(cuda_fail(h, "adjoint setup"));
 
@@ -1206,7 +1220,6 @@ int lbeh_step_adjoint(lbeh_handle *h, int nsteps, int ckpt_every, const lbeh_obs
     mom[2] = ax;
     mom[3] = bz;
   }
-  std::vector<void *> tmp;
   cudaMemsetAsync(fb[0], 0, popB, c.s);
   if (ionB) cudaMemsetAsync(nbf[0], 0, ionB, c.s);
   if (seed->f_bar) {
