@@ -268,7 +268,14 @@ int lbeh_observables_noalloc(int nx, int ny, int nz, int ncomp, int nions, int d
  * the gradients filled in.  A solve that runs out of its wait limit, or a
  * non-finite value in the forward sweep, ends the call with
  * LBEH_ERR_BARRIER_TIMEOUT or LBEH_ERR_NONFINITE and without gradients: the
- * sweep goes at most one step beyond the one in which it happened. */
+ * sweep goes at most one step beyond the one in which it happened.
+ *
+ * The call takes device memory of its own: the checkpoints, the potential of
+ * every step, one segment of states and its work arrays.  Up to 4 GB of it stay
+ * with the handle for its next call; lbeh_destroy gives them back, and so does
+ * any allocation of this library, for whichever handle, that finds no room.  A
+ * program that allocates device memory by other means and is short of it
+ * destroys the handle first.  LBEH_ERR_OOM when there is no room. */
 typedef struct lbeh_obs_seed {
   double d_deformation; /* dJ/dD of the final state */
   const double *f_bar;  /* optional [2][19][N]: dJ/df(t_end) */

@@ -117,11 +117,11 @@ Batch *batch_create(const std::vector<BatchBox> &boxes, cudaStream_t s, int *rc)
   }
   b->kern = b->K.kernel(c0.ncomp, c0.nions);
   const int nb = (int)boxes.size();
-  bool ok = cudaMalloc(&b->par, sizeof(int) * 2 * nb) == cudaSuccess;
-  ok &= cudaMalloc(&b->status, sizeof(int) * nb) == cudaSuccess;
+  bool ok = dev_alloc((void **)&b->par, sizeof(int) * 2 * nb);
+  ok &= dev_alloc((void **)&b->status, sizeof(int) * nb);
   ok &= cudaMallocHost(&b->hpar, sizeof(int) * 2 * nb) == cudaSuccess;
   ok &= cudaMallocHost(&b->hstatus, sizeof(int) * nb) == cudaSuccess;
-  ok &= cudaMalloc(&b->table, b->K.rec_bytes * nb) == cudaSuccess;
+  ok &= dev_alloc(&b->table, b->K.rec_bytes * nb);
   if (!ok) {
     batch_destroy(b);
     *rc = LBEH_ERR_OOM;
@@ -289,7 +289,7 @@ bool take(Batch *b, Snapshot &sn) {
   sn.bufs.emplace_back(b->status, sizeof(int) * b->boxes.size());
   for (auto &bf : sn.bufs) {
     void *p = nullptr;
-    if (cudaMalloc(&p, bf.second) != cudaSuccess) return false;
+    if (!dev_alloc(&p, bf.second)) return false;
     sn.copies.push_back(p);
     cudaMemcpyAsync(p, bf.first, bf.second, cudaMemcpyDeviceToDevice, b->s);
   }

@@ -16,6 +16,10 @@ namespace lbeh {
 extern std::atomic<long long> g_launches;
 inline void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
+// Device memory; where there is no room, blocks that handles keep idle between
+// their calls are freed first (kept_block.h).
+bool dev_alloc(void **p, size_t bytes);
+
 // Everything a launch needs: sizes, model constants and device pointers.
 // Field pointers are of the compute type T (double for FP64, float otherwise)
 // unless noted; populations are of the storage type of the precision mode.

@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "kept_block.h"
 
 using namespace lbeh;
 
@@ -70,12 +71,28 @@ struct lbeh_handle {
   bool stats_stale = false;  // Poisson statistics not read back since a batched step
   Poisson *adj_pois = nullptr;  // solver of the adjoint Poisson problems (created on first use)
   long long wait_limit = 0;     // barrier-wait polls of the Poisson solves (0: default)
-  void *adj_block = nullptr;    // device memory of the adjoint calls, kept between them up to kAdjKeep
-  size_t adj_block_bytes = 0;
+  KeptBlock adj_block;          // device memory of the adjoint calls, kept between them up to kAdjKeep
   int *watch = nullptr;         // pinned: status words of the last two steps of a sweep (StatusWatch)
 };
 
 std::atomic<long long> lbeh::g_launches{0};
+
+namespace {
+struct CudaMemory {
+  static bool alloc(void **p, size_t bytes) {
+    if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+    cudaGetLastError();
+    return false;
+  }
+  static void free(void *p) { cudaFree(p); }
+};
+KeptBlocks<CudaMemory> &kept_blocks() {
+  static auto *k = new KeptBlocks<CudaMemory>;  // outlives handles destroyed at exit
+  return *k;
+}
+}  // namespace
+
+bool lbeh::dev_alloc(void **p, size_t bytes) { return kept_blocks().alloc(p, bytes); }
 
 namespace {
 
@@ -143,7 +160,7 @@ struct StageTimer {
 
 void *dalloc(lbeh_handle *h, size_t bytes) {
   void *p = nullptr;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) return nullptr;
+  if (!dev_alloc(&p, bytes)) return nullptr;
   h->allocs.push_back(p);
   return p;
 }
@@ -165,7 +182,7 @@ void *stage_buf(lbeh_handle *h, size_t bytes, std::vector<void *> &tmp) {
       return b.p;
     }
   void *p = nullptr;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) return nullptr;
+  if (!dev_alloc(&p, bytes)) return nullptr;
   h->stage.push_back({p, bytes, true});
   tmp.push_back(p);
   return p;
@@ -728,7 +745,7 @@ static void destroy_handle(lbeh_handle *h) {
   if (h->ev_cp) cudaEventDestroy(h->ev_cp);
   poisson_destroy(h->pois);
   poisson_destroy(h->adj_pois);
-  if (h->adj_block) cudaFree(h->adj_block);
+  kept_blocks().drop(h->adj_block);
   if (h->watch) cudaFreeHost(h->watch);
   for (void *a : h->allocs) cudaFree(a);
   for (auto &b : h->stage) cudaFree(b.p);
@@ -1019,8 +1036,12 @@ int lbeh_observables(lbeh_handle *h, lbeh_obs *out) {
 namespace {
 // Device memory of one adjoint call, laid out in one block: a first pass over
 // the requests measures it, a second one hands out the addresses.  The handle
-// keeps a block of at most kAdjKeep bytes for its next call (25 allocations
-// and frees took 3.7 ms of a 20-step call at 96^3) and releases it at the end.
+// keeps a block of at most kAdjKeep bytes for its next call, until it is
+// destroyed or an allocation of the library needs the room (kept_block.h).
+// A 20-step call at 96^3 takes 2 GB: one allocation and free of it cost 1.6 ms
+// (30.8 ms a call against 29.1 with the block kept), 25 smaller ones 3.7.  They
+// cost in proportion to the bytes, as the call itself does; so the limit is
+// not one of time but a share, 1.4%, of the device's memory.
 constexpr size_t kAdjKeep = size_t(4) << 30;
 struct DevArena {
   char *base = nullptr;
@@ -1114,27 +1135,12 @@ int lbeh_step_adjoint(lbeh_handle *h, int nsteps, int ckpt_every, const lbeh_obs
     keep_rho = M.get(e * 2 * N), keep_eps = M.get(e * N), keep_q = M.get(e * N), keep_u = M.get(e * 3 * N);
   };
   lay_out();
-  if (h->adj_block_bytes < M.at) {
-    if (h->adj_block) cudaFree(h->adj_block);
-    h->adj_block = nullptr;
-    h->adj_block_bytes = 0;
-    if (cudaMalloc(&h->adj_block, M.at) != cudaSuccess) {
-      cudaGetLastError();
-      h->adj_block = nullptr;
-      return LBEH_ERR_OOM;
-    }
-    h->adj_block_bytes = M.at;
-  }
+  M.base = (char *)kept_blocks().take(h->adj_block, M.at);
+  if (!M.base) return LBEH_ERR_OOM;
   struct Release {
-    lbeh_handle *h;
-    ~Release() {
-      if (h->adj_block_bytes <= kAdjKeep) return;
-      cudaFree(h->adj_block);
-      h->adj_block = nullptr;
-      h->adj_block_bytes = 0;
-    }
-  } release{h};
-  M.base = (char *)h->adj_block;
+    KeptBlock &b;
+    ~Release() { kept_blocks().put(b, kAdjKeep); }
+  } release{h->adj_block};
   lay_out();
   cudaMemsetAsync(astatus, 0, sizeof(int), c.s);
 

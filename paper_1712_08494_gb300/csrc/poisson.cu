@@ -365,7 +365,7 @@ template <> std::vector<Level<float>> &levels<float>(Poisson *p) { return p->Lf;
 
 template <typename T> static T *alloc(Poisson *p, long long n) {
   void *ptr = nullptr;
-  if (cudaMalloc(&ptr, n * sizeof(T)) != cudaSuccess) return nullptr;
+  if (!dev_alloc(&ptr, n * sizeof(T))) return nullptr;
   p->allocs.push_back(ptr);
   return (T *)ptr;
 }

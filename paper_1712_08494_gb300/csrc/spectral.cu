@@ -44,7 +44,7 @@ bool spectral_supported(const Dims &d, int fp64) {
 template <typename T> static bool spectral_setup(Spectral *s, const Dims &d) {
   auto dal = [&](size_t bytes) -> void * {
     void *ptr = nullptr;
-    if (cudaMalloc(&ptr, bytes) != cudaSuccess) return nullptr;
+    if (!dev_alloc(&ptr, bytes)) return nullptr;
     s->allocs.push_back(ptr);
     return ptr;
   };

@@ -83,3 +83,29 @@ def test_adjoint_that_fails_gives_its_staging_back(program, prec):
         s.close()
         assert fake.fake_live() == 0, fake.fake_live()
     """ % prec)
+
+
+def test_idle_adjoint_memory_is_given_back(program):
+    """The memory that a handle keeps after a gradient goes to another handle
+    that finds no room, and comes back for the next gradient once there is."""
+    program("""
+        a, w = drop(n=16)
+        before = fake.fake_live()
+        assert code(a.step_adjoint, 6, 2) == lbeh.LBEH_OK
+        kept = fake.fake_live() - before
+        assert kept > 0
+        b = lbeh.System(w.params)
+        need = fake.fake_live() - kept - before  # of a second handle
+        b.close()
+        full = fake.fake_live() + need
+        fake.fake_capacity(full - 1)  # one byte too few for the handle beside the block
+        b = lbeh.System(w.params)
+        assert need < fake.fake_live() < full
+        assert code(a.step_adjoint, 6, 2) == lbeh.LBEH_ERR_OOM  # the handle in use keeps its own
+        assert a.observables().steps == 6
+        b.close()
+        assert code(a.step_adjoint, 6, 2) == lbeh.LBEH_OK
+        assert a.observables().steps == 12
+        a.close()
+        assert fake.fake_live() == 0
+    """)
