@@ -1108,10 +1108,11 @@ __device__ __forceinline__ void residual_site(const PArgs<T> &a, const Level<T> 
 
 // Four cells of a row (FP32, rows of a multiple of four cells): 16-byte loads
 // of the row and its four neighbour rows and one word past each end, 24 loads
-// instead of 22 per cell; the thread's sums take one term per four cells.
+// instead of 22 per cell.  out: the residual, rhs: the right-hand side's high
+// word, pot: the potential's high word of each cell, for the caller's sums.
 template <typename T>
 __device__ __forceinline__ void residual_quad(const PArgs<T> &a, const Level<T> &L0, int g, int y, int z, DF qbar,
-                                              float (&out)[4], float &r2, float &b2, float &ps) {
+                                              float (&out)[4], float (&rhs)[4], float (&pot)[4]) {
   const unsigned nx = unsigned(L0.nx), sz = nx * unsigned(L0.ny), n = unsigned(L0.N);
   const unsigned x0 = 4u * unsigned(g), row = unsigned(z) * sz + unsigned(y) * nx, i = row + x0;
   const unsigned rw[5] = {i, y + 1 == L0.ny ? i - (sz - nx) : i + nx, y == 0 ? i + (sz - nx) : i - nx,
@@ -1127,7 +1128,6 @@ __device__ __forceinline__ void residual_quad(const PArgs<T> &a, const Level<T> 
   const float hp = a.phi_hi[ip], hm = a.phi_hi[im], lp = a.phi_lo[ip], lm = a.phi_lo[im], ep = a.eps[ip],
               em = a.eps[im];
   const Vec<float, 4> q = ldv<4>(a.q + i);
-  r2 = b2 = ps = 0.f;
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
     const float hi[6] = {v < 3 ? h[0].v[v < 3 ? v + 1 : 3] : hp, v > 0 ? h[0].v[v > 0 ? v - 1 : 0] : hm,
@@ -1140,9 +1140,8 @@ __device__ __forceinline__ void residual_quad(const PArgs<T> &a, const Level<T> 
                          0.5f * (e0 + e[2].v[v]), 0.5f * (e0 + e[3].v[v]), 0.5f * (e0 + e[4].v[v])};
     const ResDF r = residual_df(a, q.v[v], qbar, h[0].v[v], l[0].v[v], hi, lo, kk);
     out[v] = r.r;
-    r2 += r.r * r.r;
-    b2 += r.b * r.b;
-    ps += h[0].v[v];
+    rhs[v] = r.b;
+    pot[v] = h[0].v[v];
   }
 }
 
@@ -1218,14 +1217,17 @@ __device__ bool residual_pass(const PArgs<T> &a, const Team &tm, const Level<T> 
   if constexpr (DFM) {
     if (L0.split && (L0.nx & 3) == 0) {
       const Share s = share(tm, unsigned(N >> 2));
-      for (Walk w(s.t0, s.dt, L0.nx >> 2, L0.ny); w.z < L0.nz; w.next())
-      {
-        float out[4], q2, c2, p;
-        residual_quad(a, L0, w.u, w.y, w.z, qbar_df, out, q2, c2, p);
+      for (Walk w(s.t0, s.dt, L0.nx >> 2, L0.ny); w.z < L0.nz; w.next()) {
+        float out[4], rhs[4], pot[4];
+        residual_quad(a, L0, w.u, w.y, w.z, qbar_df, out, rhs, pot);
         st_quad<float>(L0.b, unsigned(N >> 1), site32(L0.dims(), 4 * w.u, w.y, w.z) >> 1, (w.y + w.z) & 1, out);
-        sr.add(q2);
-        sb.add(c2);
-        sp.add(p);
+        // each cell's terms in double-float, as in residual_site
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          sr.add(out[v] * out[v]);
+          sb.add(rhs[v] * rhs[v]);
+          sp.add(pot[v]);
+        }
       }
     } else {
       const Share s = share(tm, unsigned(L0.N));
@@ -1272,7 +1274,6 @@ __device__ __forceinline__ void carry_quad(const PArgs<T> &a, const Level<T> &L,
   const float xp = L.x[ip], xm = L.x[im], ep = L.eps[ip], em = L.eps[im];
   ld_quad<float>(L.b, half, i, pr, b);
   Vec<float, 4> h = ldv<4>(a.phi_hi + 2u * i), l = ldv<4>(a.phi_lo + 2u * i);
-  float r2 = 0.f, ps = 0.f;
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
     const float xv[6] = {v < 3 ? x[v < 3 ? v + 1 : 3] : xp, v > 0 ? x[v > 0 ? v - 1 : 0] : xm,
@@ -1284,17 +1285,15 @@ __device__ __forceinline__ void carry_quad(const PArgs<T> &a, const Level<T> &L,
     for (int k = 0; k < 6; ++k) Ae += 0.5f * (e[v] + ev[k]) * (xv[k] - x[v]);
     const float r = b[v] - Ae;
     out[v] = r;
-    r2 += r * r;
+    sr.add(r * r);
     const DF s = df_add_f(DF{h.v[v], l.v[v]}, x[v]);
     h.v[v] = s.hi;
     l.v[v] = s.lo;
-    ps += s.hi;
+    sp.add(s.hi);
   }
   st_quad<float>(L.b, half, i, pr, out);
   stv<4>(a.phi_hi + 2u * i, h);
   stv<4>(a.phi_lo + 2u * i, l);
-  sr.add(r2);
-  sp.add(ps);
 }
 
 // the same for one cell, any layout

@@ -1060,8 +1060,14 @@ __device__ void residual_cells(const SArgs<T> &a, double qbar, DF qbar_df, doubl
       const Share s = share(tm, unsigned(d.N >> 2));
       for (Walk w(s.t0, s.dt, d.nx >> 2, d.ny); w.z < d.nz; w.next()) {
         Vec<float, 4> out;
-        float r2, b2, p;
-        residual_quad(pa, L0, w.u, w.y, w.z, qbar_df, out.v, r2, b2, p);
+        float rhs[4], pot[4], r2 = 0.f, b2 = 0.f, p = 0.f;
+        residual_quad(pa, L0, w.u, w.y, w.z, qbar_df, out.v, rhs, pot);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          r2 += out.v[v] * out.v[v];
+          b2 += rhs[v] * rhs[v];
+          p += pot[v];
+        }
         stv<4>(L0.b + site32(d, 4 * w.u, w.y, w.z), out);
         sr.add(r2);
         sb.add(b2);
