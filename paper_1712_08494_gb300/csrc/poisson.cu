@@ -554,6 +554,10 @@ Poisson *poisson_create(const Ctx &c, int fp64) {
     return p;
   }
   bool ok = fp64 ? setup<double>(p, c.d) : setup<float>(p, c.d);
+  double lo = 0.0;
+  const double hi = eps_range(c, &lo);
+  for (auto &l : p->Ld) l.far = !(lo >= 1.0 / kFarScale<double> && hi <= kFarScale<double>);
+  for (auto &l : p->Lf) l.far = !(lo >= 1.0 / kFarScale<float> && hi <= kFarScale<float>);
   if (fp64) {
     p->phi_prev = alloc<double>(p, c.d.N);
   } else {

@@ -35,6 +35,7 @@ template <typename T> struct Level {
   const T *eps = nullptr;  // set (finest split level, FP32): faces (eps_i + eps_{i+a})/2 formed from eps, k unused
   bool rb = false;         // red-black colourable: every extent even or one
   bool split = false;      // arrays stored colour by colour (below)
+  bool far = false;        // permittivities so large or small that products of faces leave the type's range
   __host__ __device__ Dims dims() const { return Dims{nx, ny, nz, N}; }
 };
 
@@ -175,8 +176,13 @@ __device__ __forceinline__ void stencil_n(const Level<T> &L, const Nbr &c, const
 // indices are compile-time constants, so the small coordinate arrays stay in
 // registers.  The series form takes one division instead of four: what bounds
 // the coarsening in FP64 is the division (the FP64 rate of the target is two
-// operations per cycle and SM), in FP32 its instruction count.
-template <typename T> __device__ __forceinline__ T series(T k_in, T k_sh, T k_nx) {
+// operations per cycle and SM), in FP32 its instruction count.  It multiplies
+// faces before it divides; boxes whose permittivities are beyond kFarScale
+// (`far`) take the sum of reciprocals.
+template <typename T> constexpr double kFarScale = 0x1p24;  // FP32: products of two faces of the coarsest level stay normal
+template <> constexpr double kFarScale<double> = 0x1p400;
+template <typename T> __device__ __forceinline__ T series(T k_in, T k_sh, T k_nx, bool far = false) {
+  if (far) return T(0.5) / (T(0.5) / k_in + T(1) / k_sh + T(0.5) / k_nx);
   const T bc = k_sh * k_nx, den = bc + k_in * (T(2) * k_nx + k_sh);
   return den > T(0) ? k_in * (bc / den) : T(0);  // 1/4 of 2 / (1/(2 k_in) + 1/k_sh + 1/(2 k_nx))
 }
@@ -213,7 +219,7 @@ __device__ __forceinline__ T coarse_coef(const Level<T> &F, const Level<T> &C, i
         const T k_sh = kf(q);
         q[AX] = x0 + 2 == fn[AX] ? 0 : x0 + 2;
         const T k_nx = kf(q);
-        acc += series(k_in, k_sh, k_nx);
+        acc += series(k_in, k_sh, k_nx, F.far);
       } else {
         acc += kf(q);
       }
@@ -1411,7 +1417,7 @@ __device__ void poisson_body(const PArgs<T> &a, const Team &tm, unsigned char *s
     const Level<T> F = lv[l - 1], C = lv[l];
     const Dims c = C.dims();
     const Share s = share(tm, unsigned(C.N));
-    const bool from_eps = F.eps && C.cf[0] && C.cf[1] && C.cf[2] && C.nx > 1 && C.ny > 1 && C.nz > 1;
+    const bool from_eps = F.eps && !F.far && C.cf[0] && C.cf[1] && C.cf[2] && C.nx > 1 && C.ny > 1 && C.nz > 1;
     for (Walk w(s.t0, s.dt, c.nx, c.ny); w.z < c.nz; w.next()) {
       const unsigned I = cell_at(C, site32(c, w.u, w.y, w.z), (w.u + w.y + w.z) & 1);
       T k[3];
