@@ -1,15 +1,17 @@
 """Host checks of the spectral transform core (csrc/spectral.cuh): the
 mixed-radix line transform against numpy's FFT, two real lines transformed
 as one complex line, the five tile passes of the device solver's plan path
-(the path of line lengths other than 32, 64, 128, 256: same tile indexing,
-line pairing and symbol scaling, natural order) as an exact inverse of eps_ref
+(the path of lines that are not transformed in registers: same tile indexing,
+line pairing and symbol scaling, natural order; here on the wide plans) as an exact inverse of eps_ref
 times the periodic seven-point Laplacian on ragged boxes and odd extents, in
 FP32 and FP64, and a conjugate-gradient solve of the oracle's
 variable-permittivity Poisson problem (Sec. II.B, II.D) preconditioned by it.
 The register passes of the other lengths are pinned lane by lane (forward
 transform into the storage order, inverse transform out of it, the split of
-two real lines from shuffled partners).  The device solver (csrc/spectral.cu)
-is compiled for sm_103a where nvcc is present."""
+two real lines from shuffled partners).  The host side of the device solver
+(csrc/spectral.cu) is compiled for sm_103a where nvcc is present; its kernel
+variants are in test_spectral_variants, the narrow line plans and the register
+DFTs in test_spectral_plans."""
 import ctypes as C
 import os
 import shutil
