@@ -14,6 +14,7 @@
 #include <utility>
 #include <vector>
 
+#include "batch_shape.h"
 #include "internal.h"
 
 namespace lbeh {
@@ -40,10 +41,11 @@ struct Batch {
   std::map<std::pair<int, int>, cudaGraphExec_t> graphs;  // (nsteps, cluster blocks)
 };
 
-static bool feasible(Batch *b, int cpb) {
+// clusters of cpb blocks that run at once (0: the shape cannot launch)
+static int active_clusters(Batch *b, int cpb) {
   if (cpb > 8 && cudaFuncSetAttribute(b->kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return 0;
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cpb);
@@ -59,10 +61,11 @@ static bool feasible(Batch *b, int cpb) {
   int n = 0;
   if (cudaOccupancyMaxActiveClusters(&n, b->kern, &cfg) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return 0;
   }
-  return n > 0;
+  return n;
 }
+static bool feasible(Batch *b, int cpb) { return active_clusters(b, cpb) > 0; }
 
 static cudaError_t launch(Batch *b, int rec0, int nrec, int nsteps, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
@@ -156,15 +159,22 @@ Batch *batch_create(const std::vector<BatchBox> &boxes, cudaStream_t s, int *rc)
     *rc = LBEH_ERR_CUDA;
     return nullptr;
   }
-  // default shape: the smallest portable cluster giving two waves of blocks
-  int dev = 0, nsm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  // default shape: the portable cluster with the least estimated time.  The
+  // rule before, the smallest cluster giving two waves of blocks, meant two
+  // blocks per SM; at one block per SM it had 64 boxes of 24^3 in clusters of 8
+  // (1317 us a step, in clusters of 2 478) and 32 of 16^3 too (384, in 4 145).
+  std::vector<long long> cells;
+  for (int t = 0; t < nb; ++t) cells.push_back(b->boxes[b->order[t]].c->d.N);
+  const double latency = c0.prec == LBEH_FP64 ? kBatchLatencyF64 : kBatchLatency;
+  double best = 0.0;
   b->cpb = 0;
   for (int cpb : kShapes) {
-    if (cpb > 8 || !feasible(b, cpb)) continue;
+    const int slots = cpb > 8 ? 0 : active_clusters(b, cpb);
+    if (slots == 0) continue;
+    const double t = batch_estimate(cells, cpb, slots, latency);
+    if (b->cpb && t >= best) continue;
     b->cpb = cpb;
-    if ((long long)cpb * nb >= 2LL * nsm) break;
+    best = t;
   }
   if (b->cpb == 0) {
     batch_destroy(b);
