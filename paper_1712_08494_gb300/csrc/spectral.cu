@@ -24,7 +24,7 @@ struct Spectral {
   int ncode = 0, ntw = 0, ns = 0;
   double eps_ref = 1.0;
   bool mix = false;  // an axis that is not 32, 64, 128 or 256
-  bool big = false;  // at least kBigCells cells, or FP64
+  bool big = false;  // the large form: large_form(), or FP64
 };
 
 static const void *variant(const Spectral *s) {
@@ -62,7 +62,7 @@ template <typename T> static bool spectral_setup(Spectral *s, const Dims &d) {
   s->e = base + 3 * stride;
   s->w = base + 4 * stride;
   const int ns[3] = {d.nx, d.ny, d.nz};
-  s->big = sizeof(T) == 8 || d.N >= kBigCells;
+  s->big = sizeof(T) == 8 || large_form(d.nx, d.ny, d.nz);
   size_t tiles = 0;
   for (int A = 0; A < 3; ++A) {
     const int n = ns[A];

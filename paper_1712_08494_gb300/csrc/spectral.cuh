@@ -290,6 +290,50 @@ inline int plan_radices(int N, int *rad, bool wide = true) {
   return 0;
 }
 
+// K of a line of N = 32 K points that one warp transforms in registers (0: by its plan's stages)
+inline int reg_fft_k(int N, bool big) {
+  const int K = N % 32 == 0 ? N / 32 : 0;
+  if (K == 1 || K == 2 || K == 4 || K == 8) return K;
+  return big && (K <= 7 || K == 10 || K == 12) ? K : 0;
+}
+
+// The form of an FP32 solve.  The large form has wide plans, register lines of
+// every K and passes on 16-byte words of cells; the small form has narrow plans
+// and K = 1, 2, 4, 8, and fewer registers in its kernel.
+//
+// Below 2^20 cells, small: solves of such boxes wait for latency and barriers.
+// Steps of 48^3 take 248 us in the small form against 267 in the large one, of
+// 81^3 413 / 436, of 128 x 128 x 48 417 / 461, of 32 x 32 x 512 364 / 408; 64^3
+// 264 / 261 and 84^3 419 / 418 are equal.  Lines of 96 would gain (96^3 473 /
+// 417), but the gradients of runs in such boxes, sums of cancelling FP32 terms,
+// move by some 1e-5 with any rounding of the solve, and keep theirs.
+//
+// From there on, large where it has something to offer: only lines of K = 1, 2,
+// 4, 8 (the words: 128^3 657 us against 681), a further K (128 x 128 x 384 1908 /
+// 1993), three stages saved over all axes (144^3 1141 / 1261), or one of a long
+// line (128 x 432 x 128 2227 / 2346; not where rows along x are no whole words).
+// Elsewhere its kernel's register passes lose more than the plans save: 128 x
+// 128 x 512 takes 2783 us in the large form against 2510 in the small one, 125 x
+// 128 x 128 885 / 794, 175^3 2732 / 2620.
+constexpr long long kLargeCells = 1LL << 20;
+inline bool large_form(int nx, int ny, int nz) {
+  if ((long long)nx * ny * nz < kLargeCells) return false;
+  int saved = 0, rad[kMaxStages];
+  bool plans = false, more = false;
+  for (int n : {nx, ny, nz}) {
+    if (reg_fft_k(n, false)) continue;
+    plans = true;
+    if (reg_fft_k(n, true)) {
+      more = true;
+      continue;
+    }
+    const int s = plan_radices(n, rad, false) - plan_radices(n, rad, true);
+    saved += s;
+    more |= s > 0 && n > 343 && nx % 4 == 0;
+  }
+  return !plans || more || saved >= 3;
+}
+
 // host: the plan and its tables in FP64 (converted to the compute type by the caller)
 template <class CodeVec, class TwVec> inline bool build_plan(int N, LinePlan &P, CodeVec &code, TwVec &tw, bool wide = true) {
   int rad[kMaxStages];

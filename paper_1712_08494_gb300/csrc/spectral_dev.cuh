@@ -46,14 +46,6 @@ constexpr int kU = 8;     // elements per thread whose loads are in flight toget
 template <typename T> constexpr double kInnerReduction = 1e-4;
 template <> constexpr double kInnerReduction<double> = 0.0;
 
-// Boxes of at least kBigCells cells take the wide line plans, the register
-// transforms of 32 K points for every K, and the passes on 16-byte words of
-// cells.  Smaller boxes (up to 101^3) keep the rounding that runs on them have
-// had: the gradients of lbeh_step_adjoint, sums of cancelling FP32 terms, move
-// by up to 6e-5 with a change of rounding anywhere in the solve, and there is
-// little to gain, since their solves wait for latency and barriers (64^3: the
-// word passes took ten steps from 1.711 to 1.703 ms; 128^3: 5.72 to 5.52).
-constexpr long long kBigCells = 1LL << 20;
 // rounding of the conjugate-gradient sums relative to their terms (FP32 per thread)
 constexpr double kSumNoise = 1e-6;
 
@@ -144,16 +136,11 @@ __device__ __forceinline__ bool sync_sums(const GridTeam &tm, double *part, int 
 // (both 1 on a stage's top lanes, so a stage is two FMAs and one complex
 // product on every lane, no select), then K - 1 of W_N^(lane kappa).
 constexpr int kLaneTw = 21;
-inline int reg_fft_k(int N, bool big) {
-  const int K = N % 32 == 0 ? N / 32 : 0;
-  if (K == 1 || K == 2 || K == 4 || K == 8) return K;
-  return big && (K <= 7 || K == 10 || K == 12) ? K : 0;
-}
 // The kernel comes in variants that hold only the code their boxes run (one
 // kernel of all of it spills: 128^3 y and z passes 5.6 and 9.1 -> 9.2 and 12
 // us).  MIX: an axis that is not 32, 64, 128 or 256 (line plans, further K).
-// BIG: at least kBigCells cells (wide plans, further K, 16-byte words of
-// cells); FP64 always.
+// BIG: the large form (wide plans, further K, 16-byte words of cells):
+// large_form(); FP64 always.
 // CALL(K) for the K of a register transform (FP64 lines end at 256).
 #define LBEH_WITH_K(T, MORE, K, CALL)                       \
   switch (K) {                                              \

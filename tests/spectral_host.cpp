@@ -123,6 +123,8 @@ extern "C" int precond_plan(void *u, int f64, int nx, int ny, int nz, double eps
 // stages of a line plan; the radices in order
 extern "C" int plan_stages(int N, int wide, int *rad) { return plan_radices(N, rad, wide); }
 
+extern "C" int box_form(int nx, int ny, int nz) { return large_form(nx, ny, nz); }
+
 // one complex line through its plan (interleaved parts)
 template <typename T> static int line(const T *in, T *out, int N, bool wide) {
   LinePlan P;

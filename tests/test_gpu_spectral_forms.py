@@ -1,0 +1,17 @@
+"""FP32 boxes of 2^20 cells and more that the spectral solve takes in its small
+form: the check of test_spectral_lengths (residual below the tolerance within
+the iterations that the contrast allows) on lines where the two forms' plans have
+as many stages, save one or two, and save one of a long line off whole words."""
+import pytest
+
+from test_spectral_lengths import test_solve_in_boxes_of_every_length as solve
+
+BOXES = [(512, 64, 32), (64, 64, 512), (16, 512, 128), (125, 128, 70), (343, 64, 48), (64, 175, 98), (128, 81, 128),
+         (375, 64, 48), (162, 128, 64)]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("box", BOXES)
+def test_small_form_of_large_boxes(lbeh, box):
+    assert box[0] * box[1] * box[2] >= 1 << 20
+    solve(lbeh, "fp32", box)

@@ -38,6 +38,7 @@ def spec(tmp_path_factory):
     for f in (lib.plan_line, lib.plan_line_f32):
         f.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.c_int]
     lib.plan_stages.argtypes = [C.c_int, C.c_int, C.c_void_p]
+    lib.box_form.argtypes = [C.c_int] * 3
     lib.precond_plan.argtypes = [C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int, C.c_double, C.c_int, C.c_int]
     return lib
 
@@ -113,3 +114,24 @@ def test_passes_invert_the_laplacian(spec, W, wide):
         assert spec.precond_plan(z64.ctypes.data, 1, nx, ny, nz, 0.3, W, wide) == 0
         res = 0.3 * _lap(z64) - (r64 - r64.mean())
         assert np.abs(res).max() < 1e-12 * np.abs(r64).max(), (nz, ny, nx)
+
+
+# steps of FP32 boxes of at least 2^20 cells, us: (small form, large form)
+FORMS = {
+    (128, 128, 128): (681, 657), (128, 128, 384): (1993, 1908), (192, 128, 128): (1065, 980),
+    (96, 96, 128): (598, 523), (144, 144, 144): (1261, 1141), (120, 120, 120): (832, 764),
+    (150, 150, 150): (1436, 1343), (105, 105, 105): (714, 701), (128, 432, 128): (2346, 2227),
+    (128, 450, 128): (2406, 2283), (504, 128, 128): (2835, 2681), (128, 128, 512): (2510, 2783),
+    (128, 512, 128): (2541, 2731), (125, 128, 128): (794, 885), (81, 128, 128): (634, 701),
+    (175, 175, 175): (2620, 2732), (512, 512, 32): (2774, 3031), (512, 16, 512): (1666, 1929),
+    (343, 64, 64): (649, 712), (375, 128, 128): (2142, 2307), (100, 128, 128): (690, 708),
+    (128, 128, 175): (1027, 1079), (270, 128, 128): (1627, 1702), (128, 225, 128): (1166, 1147),
+}
+
+
+def test_form_of_a_box(spec):
+    """Within 3% of the faster form; smaller boxes take the small form."""
+    for b, t in FORMS.items():
+        assert t[spec.box_form(*b)] <= 1.03 * min(t), b
+    for b in ((96, 96, 96), (101, 101, 101), (64, 64, 64), (32, 32, 512), (125, 64, 64)):
+        assert spec.box_form(*b) == 0, b
