@@ -96,7 +96,7 @@ template <typename T> static bool spectral_setup(Spectral *s, const Dims &d) {
     // l + 32 kappa of a register-transformed axis holds frequency
     // kappa + K bitrev5(l)
     std::vector<T> sy(n);
-    const int K = s->K[A] = reg_fft_k(n, s->big);
+    const int K = s->K[A] = reg_fft_k(n, s->big, sizeof(T) == 8);
     for (int j = 0; j < n; ++j) {
       int k = j;
       if (K) {

@@ -151,7 +151,9 @@ constexpr int kLaneTw = 21;
     default:                                                \
       if constexpr (MORE) {                                 \
         switch (K) {                                        \
-          case 3: CALL(3); break;                           \
+          case 3:                                           \
+            if constexpr (sizeof(T) == 4) { CALL(3); }      \
+            break;                                          \
           case 5: CALL(5); break;                           \
           case 6: CALL(6); break;                           \
           case 7: CALL(7); break;                           \

@@ -10,8 +10,18 @@ BOXES = [(512, 64, 32), (64, 64, 512), (16, 512, 128), (125, 128, 70), (343, 64,
          (375, 64, 48), (162, 128, 64)]
 
 
+# FP64 lines of 96, by their plan, along each axis
+FP64_96 = [(96, 32, 32), (32, 96, 32), (30, 32, 96), (96, 96, 96)]
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("box", BOXES)
 def test_small_form_of_large_boxes(lbeh, box):
     assert box[0] * box[1] * box[2] >= 1 << 20
     solve(lbeh, "fp32", box)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("box", FP64_96)
+def test_fp64_lines_of_96(lbeh, box):
+    solve(lbeh, "fp64", box)
