@@ -63,6 +63,9 @@ template <typename T> static bool spectral_setup(Spectral *s, const Dims &d) {
   s->w = base + 4 * stride;
   const int ns[3] = {d.nx, d.ny, d.nz};
   s->big = sizeof(T) == 8 || large_form(d.nx, d.ny, d.nz);
+  int dev = 0, nsm = 0, coop = 0, per = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   size_t tiles = 0;
   for (int A = 0; A < 3; ++A) {
     const int n = ns[A];
@@ -81,11 +84,15 @@ template <typename T> static bool spectral_setup(Spectral *s, const Dims &d) {
     // blocks per SM).  A tile of the x pass holds four arrays (r, q, e, p), one
     // of the y and z passes two (the next tile, or the other side of a stage);
     // 64-byte rows of 16 lines along x keep those passes on whole DRAM bursts
-    // up to lines of 384.
+    // up to lines of 384.  FP64 passes along y and z, bound by the FP64 rate of
+    // the SMs that have a tile, take fewer lines while there are fewer tiles
+    // than SMs: steps of 32 x 32 x 192 2384 -> 1859 us, of 64 x 75 x 64 2742 ->
+    // 2230, of 16 x 64 x 64 1687 -> 933, of 32^3 1143 -> 775.
     const size_t arrays = A == 0 ? 4 : 2;
     auto tile = [&](int w) { return arrays * size_t(w / 2) * (n + 1) * sizeof(C2<T>); };
     int W = 32, lg = 5;
-    while (W > 8 && tile(W) > (A == 0 ? 70 : 52) * 1024) {
+    while (W > 8 && (tile(W) > (A == 0 ? 70 : 52) * 1024 ||
+                     (sizeof(T) == 8 && A != 0 && tile_count(Grid3{d.nx, d.ny, d.nz}, A, W) < nsm))) {
       W /= 2;
       --lg;
     }
@@ -123,9 +130,6 @@ template <typename T> static bool spectral_setup(Spectral *s, const Dims &d) {
   for (int K : s->K) s->mix |= K != 1 && K != 2 && K != 4 && K != 8;
   const void *kern = variant(s);
   if (!raise_smem_limit(kern, smem)) return false;
-  int dev = 0, nsm = 0, coop = 0, per = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
   if (!coop || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kSB, smem) != cudaSuccess ||
       per < 1) {
