@@ -278,6 +278,8 @@ __device__ __forceinline__ void coarse_faces_from_eps(const T *__restrict__ eps,
     b2[ty] = two(x0, y[ty], z[2]);
     b3[ty] = two(x0, y[ty], z[3]);
   }
+  // the paths added in this order, as in the first form of the pass: the
+  // coated-drop run, whose contacts close or not by rounding, was checked on it
 #pragma unroll
   for (int ty = 0; ty < 2; ++ty) acc += path(e[0][ty].x, e[1][ty].x, b2[ty].x, b3[ty].x);
 #pragma unroll
@@ -397,7 +399,7 @@ __device__ __forceinline__ void prolong_range(const Level<T> &F, const Level<T> 
       return C.x[cell_at(C, site32(c, X, Y, Z), (X + Y + Z) & 1)];
     };
     T &xf = F.x[cell_at(F, unsigned(i), (x + y + z) & 1)];
-    if (C.cf[0] && C.cf[1] && C.cf[2]) {  // weights 27/64, 9/64, 3/64, 1/64
+    if (C.cf[0] && C.cf[1] && C.cf[2]) {  // weights 27/64, 9/64, 3/64, 1/64; one by one, as the general form adds them
       T acc = T(0.421875) * xc(0, 0, 0);
       acc += T(0.140625) * xc(1, 0, 0);
       acc += T(0.140625) * xc(0, 1, 0);

@@ -129,7 +129,7 @@ __device__ __forceinline__ bool sync_sums(const GridTeam &tm, double *part, int 
 
 // Shared memory of a block, loaded once per launch: the three axes' plans,
 // butterfly codes, twiddles and symbols; then the two tile buffers.
-// Lines of N = 32 K points (K = 1 to 8, 10, 12) are transformed in registers by
+// Lines of N = 32 K points (K = 1 to 8, 10, 12; reg_fft_k) are transformed in registers by
 // one warp (dif_regs, dit_regs below); its per-lane twiddles live in shared
 // memory: kLaneTw slots per lane and axis, the five cross-lane twiddles of the
 // decimation-in-frequency stages, the five of the decimation-in-time stages
@@ -912,8 +912,7 @@ __device__ void matvec_rows(const SArgs<T> &a, const T *z, T beta, bool first, d
 // q = A z + beta q, p = z + beta p over the team's cells; the thread's shares
 // of p.q and, for the prediction of the next residual, r.q and q.q
 template <typename T, bool DFM>
-__device__ void matvec_update(const SArgs<T> &a, const T *z, T beta, bool first, double *sh, double &pq, double &rq,
-                              double &qq) {
+__device__ void matvec_update(const SArgs<T> &a, const T *z, T beta, bool first, double &pq, double &rq, double &qq) {
   const Level<T> L0 = a.L0;
   const Dims d = L0.dims();
   const long long G = (long long)gridDim.x * blockDim.x;
@@ -1030,8 +1029,7 @@ __device__ void update_cells(const SArgs<T> &a, T al, bool he, CgAcc<T> &sr, CgA
 // residual_site in poisson_dev.cuh), two cells per thread with all their
 // loads in flight together; the thread's shares of |r|^2, |b|^2 and sum phi.
 template <bool BIG, typename T, bool DFM>
-__device__ void residual_cells(const SArgs<T> &a, double qbar, DF qbar_df, double *sh, double &ar, double &ab,
-                               double &ap) {
+__device__ void residual_cells(const SArgs<T> &a, double qbar, DF qbar_df, double &ar, double &ab, double &ap) {
   const PArgs<T> &pa = a.pa;
   const Level<T> &L0 = a.L0;
   const Dims d = L0.dims();
@@ -1290,13 +1288,13 @@ __global__ void __launch_bounds__(kSB, 2) k_spectral(SArgs<T> a) {
   const bool carry = tol >= kTrustTol;
   int it = 0;
   double bn = 0.0, rr = 0.0, shift = 0.0;
-  bool have_e = false, exact = true;
+  bool have_e = false;
   for (int outer = 0;; ++outer) {
     // exact residual r = b - A phi (FP64 / double-float), |r|^2, |b|^2, sum phi
     double r2, b2, ps;
     {
       double v[3];
-      residual_cells<BIG, T, DFM>(a, qbar, qbar_df, sh, v[0], v[1], v[2]);
+      residual_cells<BIG, T, DFM>(a, qbar, qbar_df, v[0], v[1], v[2]);
       put_block_sums<3>(tm, v, pa.part, nb, sh);
       if (!sync_sums<3>(tm, pa.part, nb, v, sh)) return;
       r2 = v[0];
@@ -1305,7 +1303,6 @@ __global__ void __launch_bounds__(kSB, 2) k_spectral(SArgs<T> a) {
     }
     if (outer == 0) bn = b2;
     rr = bcast0(t0 ? rel_res(r2, bn) : 0.0, &bc[1]);
-    exact = true;
     shift = bcast0(t0 ? ps / double(N) : 0.0, &bc[2]);
     have_e = false;
     if (rr < tol || it >= max_iter || !isfinite(rr)) break;
@@ -1334,7 +1331,6 @@ __global__ void __launch_bounds__(kSB, 2) k_spectral(SArgs<T> a) {
         sum_e = v[1];
         ++it;
         rr = bcast0(t0 ? rel_res(r2, bn) : 0.0, &bc[3]);
-        exact = false;
         if (rr < target || it >= max_iter || !isfinite(rr)) break;
         // mispredicted: the x pass of the updated r
         if (!MIX || a.xrows) {
@@ -1381,7 +1377,6 @@ __global__ void __launch_bounds__(kSB, 2) k_spectral(SArgs<T> a) {
         r2 = rz[1];
         sum_e = rz[2];
         rr = bcast0(t0 ? rel_res(r2, bn) : 0.0, &bc[3]);
-        exact = false;
         if (rr < target || it >= max_iter || !isfinite(rr)) break;
       }
       const double beta = bcast0(t0 && !first ? rho / rho_old : 0.0, &bc[4]);
@@ -1390,7 +1385,7 @@ __global__ void __launch_bounds__(kSB, 2) k_spectral(SArgs<T> a) {
         double v[3];
         constexpr int W = 16 / sizeof(T);
         if (BIG && d.nx % W == 0) matvec_rows<T, W>(a, a.w, T(beta), first, v[0], v[1], v[2]);
-        else matvec_update<T, DFM>(a, a.w, T(beta), first, sh, v[0], v[1], v[2]);
+        else matvec_update<T, DFM>(a, a.w, T(beta), first, v[0], v[1], v[2]);
         put_block_sums<3>(tm, v, pa.part, nb, sh);
       }
       double fs[3];
@@ -1510,7 +1505,6 @@ __global__ void __launch_bounds__(kSB, 2) k_spectral(SArgs<T> a) {
     if (fail) atomicOr(pa.status, ST_POISSON);
     if (!isfinite(rr)) atomicOr(pa.status, ST_NONFINITE);
   }
-  (void)exact;
 }
 
 }  // namespace
